@@ -304,8 +304,8 @@ int dms_diagram_d1(const float* f, const uint32_t* order, const uint64_t* rec, d
  *                device (both read during the call).
  *   tile_variant gradient variant, 0..dms_batch_tile_variants()-1: tile shape
  *                variant % 3 (32 x 24, 32 x 16, 32 x 32 anchors per CTA) and
- *                lanes per vertex 1 + variant / 3 (two: the lane pair splits
- *                the rank comparisons, link edges and tet keys of a vertex);
+ *                threads per anchor 1 + variant / 3 (two: they split the
+ *                seven edges of an anchor);
  *                an autotuner picks one; all give the same results.
  *   order, desc, rec  concatenated outputs as in dms_order/dms_gradient, each
  *                field with its own local order and records.

@@ -3,7 +3,7 @@
 ``Batch`` owns every device buffer for one fixed list of field shapes, so a
 call allocates nothing and synchronises nothing: it can be captured once in a
 CUDA graph and replayed for each new batch of inputs.  ``autotune`` picks the
-gradient variant -- tile shape and lanes per vertex -- for a list of shapes
+gradient variant -- tile shape and threads per anchor -- for a list of shapes
 by timing the compiled variants and keeps the winner in a small JSON cache.  ``per_field`` runs the same fields
 one at a time through the single-field entry points (the comparison point for
 the batched path).
@@ -181,12 +181,12 @@ def _key(shapes, device):
 
 
 def variant_name(v: int) -> str:
-    """The gradient variant v: anchors per CTA tile and lanes per vertex."""
-    return f"32x{(24, 16, 32)[v % 3]}, {1 + v // 3} lane(s)/vertex"
+    """The gradient variant v: anchors per CTA tile and threads per anchor."""
+    return f"32x{(24, 16, 32)[v % 3]}, {1 + v // 3} thread(s)/anchor"
 
 
 def autotune(shapes, device="cuda", fields=None, reps: int = 3, use_cache: bool = True):
-    """Best gradient variant (tile shape x lanes per vertex) for these shapes,
+    """Best gradient variant (tile shape x threads per anchor) for these shapes,
     timed on the device with CUDA events over graph replays of the whole
     batch; cached by device name and shape list.  The times of the last
     call (ms per variant) are left in ``autotune.last``."""
