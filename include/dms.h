@@ -319,13 +319,12 @@ int dms_diagram_d1(const float* f, const uint32_t* order, const uint64_t* rec, d
  *                (1 << DMS_ERR_CAPACITY); the call can then be repeated with
  *                larger capacities).
  *   ws           at least dms_batch_workspace_size(...) bytes.
- * The spanning forest takes a fixed 40 Boruvka rounds (enough: the active
- * components at least halve per round); the pairing runs
- * dms_batch_max_rounds() exact rounds and finishes the saddles still live
- * in increasing weight (Alg. 1's own order): up to 4096 of them in one CTA,
- * more after a device-wide sort by one thread, which is slow when very many
- * are left (a chain of components that the exact rounds merge one per
- * round) but exact.
+ * The spanning forest and the exact rounds run on the device until no saddle
+ * is live, a round removes under 1/64 of them, or dms_batch_max_rounds() exact
+ * rounds have run; the saddles still live are finished in increasing weight
+ * (Alg. 1's own order): up to 4096 of them in one CTA, more after a
+ * device-wide sort by one thread, which is slow when very many are left (a
+ * chain of components that the exact rounds merge one per round) but exact.
  */
 int32_t dms_batch_tile_variants(void);
 int32_t dms_batch_max_rounds(void);

@@ -696,24 +696,10 @@ __device__ __forceinline__ uint32_t find_root(Nodes nd, uint32_t x) {
   return x;
 }
 
-__global__ void round_find(const uint32_t* __restrict__ live, const unsigned int* __restrict__ live_n,
-                           Tri T, Nodes nd, uint64_t round) {
-  unsigned int n = *live_n;
-  for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    uint32_t i = live[j];
-    // roots only ever gain parents: search from last round's roots
-    uint32_t a = find_root(nd, round == 1 ? T.s[i].na : T.s[i].ra);
-    uint32_t b = find_root(nd, round == 1 ? T.s[i].nb : T.s[i].rb);
-    T.s[i].ra = a;
-    T.s[i].rb = b;
-    if (a == b) continue;
-    unsigned long long tv = (round << 44) | (kMask44 - T.s[i].w);
-    if (a != nd.immortal) atomicMax(nd.best + a, tv);
-    if (b != nd.immortal) atomicMax(nd.best + b, tv);
-  }
-}
-
-// Merge rules, each exact (see the header comment):
+// ---------------------------------------------------------------------------
+// The pairing rounds.
+//
+// Merge rules of the exact rounds (see the header comment):
 //  * mutual: the saddle is the lightest live saddle of both components -> the
 //    younger root dies;
 //  * downhill: the saddle is the lightest live saddle of component a and the
@@ -723,51 +709,8 @@ __global__ void round_find(const uint32_t* __restrict__ live, const unsigned int
 //    b's root, which is older than a's, so a's root is the younger one.
 // A root dies through its own lightest saddle only, so it dies at most once
 // per round, and the links never form a cycle (each points to an older root).
-__global__ void __launch_bounds__(256) round_merge(const uint32_t* __restrict__ live,
-                                                   const unsigned int* __restrict__ live_n, Tri T,
-                                                   Nodes nd, uint64_t round, uint32_t* next,
-                                                   unsigned int* next_n) {
-  __shared__ CtaAppend sh;
-  const unsigned int n = *live_n;
-  // CTA-uniform passes: every thread reaches the appends
-  for (unsigned int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
-    const unsigned int j = base + threadIdx.x;
-    bool wait = false;
-    uint32_t i = 0;
-    if (j < n) {
-      i = live[j];
-      const uint32_t a = T.s[i].ra, b = T.s[i].rb;
-      if (a != b) {  // else both ends already joined: no pair (Alg. 1, r0 == r1)
-        const unsigned long long tv = (round << 44) | (kMask44 - T.s[i].w);
-        const bool la = a != nd.immortal && nd.best[a] == tv;
-        const bool lb = b != nd.immortal && nd.best[b] == tv;
-        uint32_t young = kNone, old = kNone;
-        if (la || lb) {
-          const uint64_t ga = nd.age[a], gb = nd.age[b];
-          if (la && lb) {
-            young = ga > gb ? a : b;
-            old = young == a ? b : a;
-          } else if (la && ga > gb) {
-            young = a;
-            old = b;
-          } else if (lb && gb > ga) {
-            young = b;
-            old = a;
-          }
-        }
-        if (young != kNone) {
-          nd.parent[young] = old;
-          T.s[i].res = young;
-        } else {
-          wait = true;  // the lightest live saddle of neither side, or uphill: wait
-        }
-      }
-    }
-    cta_append2(sh, wait, next, next_n, false, next, next_n, i);
-  }
-}
-
-// Minimum spanning forest first (Borůvka), then the pairing on its edges.
+//
+// The minimum spanning forest first (Borůvka), then the pairing on its edges:
 // Alg. 1 pairs nothing at a saddle whose ends are already joined by lighter
 // saddles, and such a saddle changes no component: these are exactly the
 // saddles outside the minimum spanning forest of the extremum graph
@@ -777,9 +720,105 @@ __global__ void __launch_bounds__(256) round_merge(const uint32_t* __restrict__ 
 // saddle is a forest edge by the cut property), with no regard to ages, so
 // components at least halve per round and the saddles inside a component
 // drop out as loops.  The exact rounds then run on the forest's edges only.
+// ---------------------------------------------------------------------------
+
+// both roots of a live saddle, and the saddle as the lightest of each so far
+__device__ __forceinline__ void find_saddle(const Tri& T, const Nodes& nd, uint32_t i,
+                                            unsigned int round) {
+  // roots only ever gain parents: search from last round's roots
+  const uint32_t a = find_root(nd, round == 1 ? T.s[i].na : T.s[i].ra);
+  const uint32_t b = find_root(nd, round == 1 ? T.s[i].nb : T.s[i].rb);
+  T.s[i].ra = a;
+  T.s[i].rb = b;
+  if (a == b) return;
+  const unsigned long long tv = ((unsigned long long)round << 44) | (kMask44 - T.s[i].w);
+  if (a != nd.immortal) atomicMax(nd.best + a, tv);
+  if (b != nd.immortal) atomicMax(nd.best + b, tv);
+}
+
+// whether a live saddle is the lightest of its roots (la, lb); false where
+// they are one (inside a component: no forest edge, no pair).  ONE: within one
+// launch, the tags are read from L2, where the atomics put them
+template <bool ONE>
+__device__ __forceinline__ bool lightest(const Tri& T, const Nodes& nd, uint32_t i, unsigned int round,
+                                         uint32_t& a, uint32_t& b, bool& la, bool& lb) {
+  a = T.s[i].ra;
+  b = T.s[i].rb;
+  if (a == b) return false;
+  const unsigned long long tv = ((unsigned long long)round << 44) | (kMask44 - T.s[i].w);
+  la = a != nd.immortal && (ONE ? __ldcg(nd.best + a) : nd.best[a]) == tv;
+  lb = b != nd.immortal && (ONE ? __ldcg(nd.best + b) : nd.best[b]) == tv;
+  return true;
+}
+
+// Borůvka: the saddle is a forest edge (tree), stays live (wait), or neither
+template <bool ONE>
+__device__ __forceinline__ void hook_saddle(const Tri& T, const Nodes& nd, uint32_t i,
+                                            unsigned int round, bool& wait, bool& tree) {
+  uint32_t a, b;
+  bool la, lb;
+  if (!lightest<ONE>(T, nd, i, round, a, b, la, lb)) return;
+  tree = la || lb;
+  wait = !tree;
+  // each component hooks under the other end of its own lightest saddle; two
+  // components that chose the same saddle hook one way only
+  if (la && lb) nd.parent[min(a, b)] = max(a, b);
+  else if (la) nd.parent[a] = b;
+  else if (lb) nd.parent[b] = a;
+}
+
+// exact round: the saddle kills a root, stays live (wait), or neither
+template <bool ONE>
+__device__ __forceinline__ void merge_saddle(const Tri& T, const Nodes& nd, uint32_t i,
+                                             unsigned int round, bool& wait) {
+  uint32_t a, b;
+  bool la, lb;
+  if (!lightest<ONE>(T, nd, i, round, a, b, la, lb)) return;
+  uint32_t young = kNone, old = kNone;
+  if (la || lb) {
+    const uint64_t ga = nd.age[a], gb = nd.age[b];
+    if (la && (lb || ga > gb)) {
+      young = ga > gb ? a : b;
+      old = ga > gb ? b : a;
+    } else if (lb && gb > ga) {
+      young = b;
+      old = a;
+    }
+  }
+  wait = young == kNone;  // the lightest of neither side, or uphill: wait
+  if (!wait) {
+    nd.parent[young] = old;
+    T.s[i].res = young;
+  }
+}
+
+// ---- one launch per phase: rounds of many saddles
+__global__ void round_find(const uint32_t* __restrict__ live, const unsigned int* __restrict__ live_n,
+                           Tri T, Nodes nd, unsigned int round) {
+  const unsigned int n = *live_n;
+  for (unsigned int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    find_saddle(T, nd, live[j], round);
+}
+
+__global__ void __launch_bounds__(256) round_merge(const uint32_t* __restrict__ live,
+                                                   const unsigned int* __restrict__ live_n, Tri T,
+                                                   Nodes nd, unsigned int round, uint32_t* next,
+                                                   unsigned int* next_n) {
+  __shared__ CtaAppend sh;
+  const unsigned int n = *live_n;
+  // CTA-uniform passes: every thread reaches the appends
+  for (unsigned int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
+    const unsigned int j = base + threadIdx.x;
+    bool wait = false;
+    const uint32_t i = j < n ? live[j] : 0;
+    if (j < n) merge_saddle<false>(T, nd, i, round, wait);
+    cta_append2(sh, wait, next, next_n, false, next, next_n, i);
+  }
+}
+
 __global__ void __launch_bounds__(256) boruvka_hook(const uint32_t* __restrict__ live,
                                                     const unsigned int* __restrict__ live_n, Tri T,
-                                                    Nodes nd, uint64_t round, uint32_t* next,
+                                                    Nodes nd, unsigned int round, uint32_t* next,
                                                     unsigned int* next_n, uint32_t* forest,
                                                     unsigned int* forest_n) {
   __shared__ CtaAppend sh;
@@ -788,36 +827,233 @@ __global__ void __launch_bounds__(256) boruvka_hook(const uint32_t* __restrict__
   for (unsigned int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
     const unsigned int j = base + threadIdx.x;
     bool wait = false, tree = false;
-    uint32_t i = 0;
-    if (j < n) {
-      i = live[j];
-      const uint32_t a = T.s[i].ra, b = T.s[i].rb;
-      if (a != b) {  // else inside one component: not a forest edge
-        const unsigned long long tv = (round << 44) | (kMask44 - T.s[i].w);
-        const bool sa = a != nd.immortal && nd.best[a] == tv;
-        const bool sb = b != nd.immortal && nd.best[b] == tv;
-        if (!sa && !sb) {
-          wait = true;
-        } else {
-          tree = true;
-          // each component hooks under the other end of its own lightest
-          // saddle; two components that chose the same saddle hook one way only
-          if (sa && sb) nd.parent[min(a, b)] = max(a, b);
-          else if (sa) nd.parent[a] = b;
-          else nd.parent[b] = a;
-        }
-      }
-    }
+    const uint32_t i = j < n ? live[j] : 0;
+    if (j < n) hook_saddle<false>(T, nd, i, round, wait, tree);
     cta_append2(sh, wait, next, next_n, tree, forest, forest_n, i);
   }
 }
 
-__global__ void reset_nodes(Nodes nd, int64_t nnode) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nnode;
+// node arrays back to singletons: *n_dev + n nodes (n_dev may be null)
+__global__ void reset_nodes(Nodes nd, const int64_t* __restrict__ n_dev, int64_t n) {
+  if (n_dev) n += *n_dev;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     nd.parent[i] = (uint32_t)i;
     nd.best[i] = 0ull;
   }
+}
+
+// ---- all rounds in one launch: fewer saddles
+// A cooperative grid (all its CTAs resident) takes its counts from device
+// memory and meets at a barrier after each phase, so that no round costs a
+// launch or a read of a count on the host; when few saddles are live, CTA 0
+// goes on alone.  A round cost 25-30 us with one launch per phase and a
+// synchronising read, 4 us with the grid barrier, 3 us in the lone CTA: the
+// D0/D2 stage of 24^3 and 64^3 mixtures 733 -> 446 and 1119 -> 765 us, of 2 M
+// vertices of noise 2.5 -> 1.4 ms, of a 1501 x 999 image 3.8 -> 1.1 ms (its
+// last 4096 saddles used to go to the one-thread finish).  Many saddles hide
+// the launches, and the grid's static share per CTA costs more: with all
+// rounds in here the stage took 92.4 instead of 89.4 ms on the 1024^3 mixture
+// (117 M saddles) and 31.4 instead of 30.5 ms on 512^3 quantised noise; the
+// line lies where both ways cost the same (512 K to 10 M: within 1 %).
+constexpr int kRoundThreads = 512;
+constexpr unsigned int kSolo = 4096;           // live saddles that CTA 0 works alone
+constexpr int64_t kSoloNodes = 1 << 16;        // nodes that it sets back alone
+constexpr int64_t kOneLaunch = (int64_t)3 << 20;  // saddles up to which the rounds are one launch
+constexpr unsigned int kMaxExactRounds = 256;  // then the sorted finish, whatever is left
+constexpr unsigned int kMaxForestRounds = 64;  // components at least halve per round
+constexpr uint32_t kBarrierPolls = 1u << 23;
+
+// words of DiagWs::ctr
+enum : int {
+  kCtrLive = 0,      // saddles live after the walks
+  kCtrNext = 1,      // live saddles of the rounds of one launch per phase: with kCtrLive in turn
+  kCtrForest = 2,    // saddles of the spanning forest
+  kCtrChanged = 3,   // (self-correcting pairing)
+  kCtrBig = 4,       // saddles left to the device-wide sorted finish (batch)
+  kCtrWalk = 6,      // walk cursor
+  kCtrRound = 8,     // three live counts in turn
+  kCtrLeft = 11,     // saddles left live by the exact rounds
+  kCtrBarrier = 12,
+  kCtrAbort = 13,
+  kCtrWords = 16
+};
+
+struct Rounds {
+  Tri T;
+  Nodes nd;
+  uint32_t *cur, *nxt;   // the live saddles, room for the next round's
+  const unsigned int* n;  // their count
+  unsigned int round;     // the first round's number
+  // Borůvka rounds append the forest's saddles to `forest` (null: exact
+  // rounds); then, unless forest_only, the exact rounds on them follow
+  uint32_t* forest;
+  bool forest_only;
+  bool first_found;       // the first round's search is done (link_walks)
+  unsigned int* ctr;
+  const int64_t* n_dev;   // node count: *n_dev + nnode, or nnode alone
+  int64_t nnode;
+  uint32_t* left;         // the saddles that the exact rounds leave live end here
+};
+
+// as cta_append2, for kRoundThreads
+struct RoundAppend {
+  unsigned int off[2][kRoundThreads / 32];
+  unsigned int base[2];
+};
+__device__ __forceinline__ void round_append2(RoundAppend& sh, bool w0, uint32_t* l0, unsigned int* c0,
+                                              bool w1, uint32_t* l1, unsigned int* c1, uint32_t v) {
+  constexpr int NW = kRoundThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned b0 = __ballot_sync(0xFFFFFFFFu, w0), b1 = __ballot_sync(0xFFFFFFFFu, w1);
+  if (lane == 0) {
+    sh.off[0][warp] = __popc(b0);
+    sh.off[1][warp] = __popc(b1);
+  }
+  __syncthreads();
+  if (warp < 2) {
+    const unsigned int x = lane < NW ? sh.off[warp][lane] : 0u;
+    unsigned int t = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int y = __shfl_up_sync(0xFFFFFFFFu, t, o);
+      if (lane >= o) t += y;
+    }
+    if (lane < NW) sh.off[warp][lane] = t - x;
+    if (lane == 31) sh.base[warp] = t ? atomicAdd(warp ? c1 : c0, t) : 0u;
+  }
+  __syncthreads();
+  const unsigned lt = (1u << lane) - 1u;
+  if (w0) l0[sh.base[0] + sh.off[0][warp] + __popc(b0 & lt)] = v;
+  if (w1) l1[sh.base[1] + sh.off[1][warp] + __popc(b1 & lt)] = v;
+  __syncthreads();
+}
+
+// all CTAs of the grid (CTA 0 alone once solo); false when the others did not
+// arrive within kBarrierPolls polls or gave up themselves
+__device__ __forceinline__ bool round_sync(unsigned int* ctr, unsigned int& epoch, bool solo) {
+  __syncthreads();
+  if (solo) return true;
+  int ok = 1;
+  ++epoch;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(ctr + kCtrBarrier, 1u);
+    volatile unsigned int* bar = ctr + kCtrBarrier;
+    volatile unsigned int* stop = ctr + kCtrAbort;
+    const unsigned int want = epoch * gridDim.x;
+    uint32_t it = 0;
+    while ((int)(*bar - want) < 0) {
+      if (++it > kBarrierPolls || *stop) {
+        *stop = 1;
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// An exact round that removes under 1/64 of the live saddles (a chain of
+// components merging one saddle per round, say), or the round limit, ends the
+// rounds: what is left (ctr[kCtrLeft] saddles, in `left`) goes to the sorted
+// finish, which continues Alg. 1 exactly for any number of saddles.
+__global__ void __launch_bounds__(kRoundThreads, 4) pair_rounds(const Rounds R, int32_t* dstatus) {
+  __shared__ RoundAppend sh;
+  unsigned int* const ctr = R.ctr;
+  const Tri T = R.T;
+  const Nodes nd = R.nd;
+  const int64_t nn = (R.n_dev ? *R.n_dev : 0) + R.nnode;
+  unsigned int epoch = 0, round = R.round;
+  unsigned int n = __ldcg(R.n);
+  uint32_t *cur = R.cur, *nxt = R.nxt;
+  bool solo = gridDim.x == 1, forest = R.forest != nullptr, found = R.first_found;
+  for (;;) {
+    // (many nodes are set back by the whole grid)
+    if (!solo && n <= kSolo && (!forest || nn <= kSoloNodes)) {
+      if (blockIdx.x != 0) return;
+      solo = true;
+    }
+    const unsigned int first = (solo ? 0 : blockIdx.x * kRoundThreads) + threadIdx.x;
+    const unsigned int step = solo ? kRoundThreads : gridDim.x * kRoundThreads;
+    if (n == 0) {
+      if (!forest || R.forest_only) return;
+      // the forest is complete: single components again, its saddles live
+      forest = false;
+      for (int64_t i = first; i < nn; i += step) {
+        nd.parent[i] = (uint32_t)i;
+        nd.best[i] = 0ull;
+      }
+      n = __ldcg(ctr + kCtrForest);
+      if (first < 3) ctr[kCtrRound + first] = 0;
+      nxt = R.cur;
+      cur = R.forest;
+      round = 1;
+      if (!round_sync(ctr, epoch, solo)) break;
+      continue;
+    }
+    if (forest && round > kMaxForestRounds) break;
+    if (!found) {
+      for (unsigned int j = first; j < n; j += step) find_saddle(T, nd, cur[j], round);
+      if (!round_sync(ctr, epoch, solo)) break;
+    }
+    found = false;
+    // round r counts in word r % 3; word (r + 1) % 3 was last read two rounds ago
+    unsigned int* const nxt_n = ctr + kCtrRound + round % 3;
+    if (first == 0) ctr[kCtrRound + (round + 1) % 3] = 0;
+    // CTA-uniform passes: every thread reaches the appends
+    for (unsigned int base = first - threadIdx.x; base < n; base += step) {
+      const unsigned int j = base + threadIdx.x;
+      bool wait = false, tree = false;
+      const uint32_t i = j < n ? cur[j] : 0;
+      if (j < n) {
+        if (forest) hook_saddle<true>(T, nd, i, round, wait, tree);
+        else merge_saddle<true>(T, nd, i, round, wait);
+      }
+      round_append2(sh, wait, nxt, nxt_n, tree, R.forest, ctr + kCtrForest, i);
+    }
+    if (!round_sync(ctr, epoch, solo)) break;
+    const unsigned int left = __ldcg(nxt_n);
+    uint32_t* const t = cur;
+    cur = nxt;
+    nxt = t;
+    ++round;
+    if (!forest && left && ((uint64_t)left * 64 > (uint64_t)n * 63 || round > kMaxExactRounds)) {
+      for (unsigned int j = first; j < left; j += step) R.left[j] = cur[j];
+      if (first == 0) ctr[kCtrLeft] = left;
+      return;
+    }
+    n = left;
+  }
+  // a barrier that ran out, or a forest that does not end
+  if (threadIdx.x == 0) set_status(dstatus, DMS_ERR_TIMEOUT);
+}
+
+// launches pair_rounds for at most n live saddles (its own words of ctr are
+// zero: all from kCtrRound on)
+int launch_rounds(const Rounds& R, int64_t n, int32_t* dstatus, cudaStream_t s) {
+  static int blocks = 0;
+  if (blocks == 0) {
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_rounds, kRoundThreads, 0) !=
+            cudaSuccess ||
+        per_sm < 1)
+      return DMS_ERR_CUDA;
+    blocks = sms * per_sm;
+  }
+  const unsigned grid =
+      n <= (int64_t)kSolo ? 1u
+                          : (unsigned)std::min<int64_t>(blocks, (n + kRoundThreads - 1) / kRoundThreads);
+  Rounds r = R;
+  void* args[2] = {&r, &dstatus};
+  if (cudaLaunchCooperativeKernel((const void*)pair_rounds, dim3(grid), dim3(kRoundThreads), args, 0,
+                                  s) != cudaSuccess)
+    return DMS_ERR_CUDA;
+  count_launch();
+  return DMS_OK;
 }
 
 // The last few live saddles, processed one by one in increasing weight: the
@@ -973,7 +1209,7 @@ struct DiagWs {
   Tri T0, T2;
   uint32_t *live0, *live1;
   uint32_t* forest;  // the spanning-forest saddles found by the Borůvka rounds
-  unsigned int* ctr;  // [0..1] live counts, [2] forest count, [3] changed, [4] finish count, [6] walk cursor
+  unsigned int* ctr;  // counts (kCtr...)
   Nodes nd;  // union-find nodes: parent, best live saddle, age
   // the self-correcting pairing's next links (the current ones live in
   // nd.parent and nd.best)
@@ -998,7 +1234,7 @@ DiagWs carve_diag(void* base, const int64_t* nc, int64_t nclaim) {
   w.live0 = c.take<uint32_t>(nsad);
   w.live1 = c.take<uint32_t>(nsad);
   w.forest = c.take<uint32_t>(nsad);
-  w.ctr = c.take<unsigned int>(8);
+  w.ctr = c.take<unsigned int>(kCtrWords);
   w.nd.parent = c.take<uint32_t>(nnode);
   w.nd.best = c.take<unsigned long long>(nnode);
   w.nd.age = c.take<uint64_t>(nnode);
@@ -1012,79 +1248,102 @@ DiagWs carve_diag(void* base, const int64_t* nc, int64_t nclaim) {
   return w;
 }
 
-constexpr unsigned int kSeqMax = 4096;  // live saddles left to the sequential finish
-constexpr uint64_t kMaxExactRounds = 256;  // then the sorted finish, whatever is left
-
-// the exact rounds over the live list (cur, *cur_n), alternating with (nxt, *nxt_n).
-// A round that removes under 1/64 of the live saddles (a chain of components
-// merging one saddle per round, say) or the round limit hands what is left
-// to the sorted finish at once: it continues Alg. 1 exactly for any number
-// of saddles, so the number of host-synchronised rounds stays bounded.
-int run_rounds_from(DiagWs& w, Tri T, uint32_t* cur, unsigned int* cur_n, uint32_t* nxt,
-                    unsigned int* nxt_n, cudaStream_t s, int32_t* dstatus) {
-  unsigned int prev = 0xFFFFFFFFu;
-  for (uint64_t round = 1;; ++round) {
-    unsigned int h = 0;
-    DMS_CUDA_OK(cudaMemcpyAsync(&h, cur_n, sizeof(h), cudaMemcpyDeviceToHost, s));
-    DMS_CUDA_OK(cudaStreamSynchronize(s));
-    if (h == 0) break;
-    const bool stalled = (uint64_t)h * 4 > (uint64_t)prev * 3;     // < 1/4 removed
-    const bool crawling = (uint64_t)h * 64 > (uint64_t)prev * 63;  // < 1/64 removed
-    if ((h <= kSeqMax && stalled) || crawling || round >= kMaxExactRounds) {
-      // few saddles left and the rounds have stalled, or no real progress:
-      // finish in sorted order
-      unsigned int blocks = (h + 255) / 256;
-      gather_live<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.rb.ka, w.rb.va); count_launch();
-      bool in_a = radix64::sort(w.rb, h, 44, s);
-      sequential_finish<<<1, 32, 0, s>>>(in_a ? w.rb.va : w.rb.vb, cur_n, T, w.nd); count_launch();
-      break;
-    }
-    prev = h;
-    unsigned int blocks = (unsigned int)std::min<int64_t>((h + 255) / 256, 1 << 16);
-    DMS_CUDA_OK(cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s));
-    round_find<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round); count_launch();
-    round_merge<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n); count_launch();
-    std::swap(cur, nxt);
-    std::swap(cur_n, nxt_n);
-  }
-  (void)dstatus;
+// the saddles that the rounds left live, if any, in sorted order
+int finish_sorted(DiagWs& w, Tri T, cudaStream_t s) {
+  unsigned int h = 0;
+  DMS_CUDA_OK(cudaMemcpyAsync(&h, w.ctr + kCtrLeft, sizeof(h), cudaMemcpyDeviceToHost, s));
+  DMS_CUDA_OK(cudaStreamSynchronize(s));
+  if (h == 0) return DMS_OK;
+  gather_live<<<(h + 255) / 256, 256, 0, s>>>(w.live1, w.ctr + kCtrLeft, T, w.rb.ka, w.rb.va); count_launch();
+  const bool in_a = radix64::sort(w.rb, h, 44, s);
+  sequential_finish<<<1, 32, 0, s>>>(in_a ? w.rb.va : w.rb.vb, w.ctr + kCtrLeft, T, w.nd); count_launch();
   return launch_status();
 }
 
-int run_rounds(DiagWs& w, Tri T, cudaStream_t s, int32_t* dstatus) {
-  return run_rounds_from(w, T, w.live0, w.ctr + 0, w.live1, w.ctr + 1, s, dstatus);
-}
-
-// Borůvka rounds over the live saddles in w.live0 (count ctr[0]) collect
-// the spanning forest's saddles; the node arrays are then reset and the
-// exact rounds pair the forest's saddles.
-int run_pairing(DiagWs& w, Tri T, int64_t nnode, cudaStream_t s, int32_t* dstatus,
-                bool first_found = false) {
-  uint32_t* cur = w.live0;
-  uint32_t* nxt = w.live1;
-  unsigned int* cur_n = w.ctr + 0;
-  unsigned int* nxt_n = w.ctr + 1;
-  unsigned int* forest_n = w.ctr + 2;
-  DMS_CUDA_OK(cudaMemsetAsync(forest_n, 0, sizeof(unsigned int), s));
-  for (uint64_t round = 1;; ++round) {
-    unsigned int h = 0;
-    DMS_CUDA_OK(cudaMemcpyAsync(&h, cur_n, sizeof(h), cudaMemcpyDeviceToHost, s));
-    DMS_CUDA_OK(cudaStreamSynchronize(s));
-    if (h == 0) break;
-    if (round >= 64) return DMS_ERR_TIMEOUT;  // components at least halve per round
-    const unsigned int blocks = (unsigned int)std::min<int64_t>((h + 255) / 256, 1 << 16);
+// rounds of one launch per phase while more than kOneLaunch saddles are live:
+// cur/nxt with the counts cur_n/nxt_n in turn, from `round` on; forest: the
+// Borůvka rounds
+int run_large(DiagWs& w, Tri T, uint32_t*& cur, unsigned int*& cur_n, uint32_t*& nxt,
+              unsigned int*& nxt_n, unsigned int& round, unsigned int h, bool forest, bool found,
+              cudaStream_t s) {
+  while ((int64_t)h > kOneLaunch) {
+    if (round > kMaxForestRounds) return forest ? DMS_ERR_TIMEOUT : DMS_OK;
+    const unsigned int prev = h;
+    const unsigned int blocks = std::min((h + 255) / 256, 1u << 16);
     DMS_CUDA_OK(cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s));
-    if (round > 1 || !first_found) {  // else link_walks did round 1's search
+    if (!found) {
       round_find<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round); count_launch();
     }
-    boruvka_hook<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n, w.forest, forest_n); count_launch();
+    found = false;
+    if (forest) {
+      boruvka_hook<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n, w.forest,
+                                          w.ctr + kCtrForest); count_launch();
+    } else {
+      round_merge<<<blocks, 256, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n); count_launch();
+    }
     std::swap(cur, nxt);
     std::swap(cur_n, nxt_n);
+    ++round;
+    DMS_CUDA_OK(cudaMemcpyAsync(&h, cur_n, sizeof(h), cudaMemcpyDeviceToHost, s));
+    DMS_CUDA_OK(cudaStreamSynchronize(s));
+    if (!forest && (uint64_t)h * 64 > (uint64_t)prev * 63) break;  // pair_rounds will end, too
   }
-  const unsigned int nb = (unsigned int)std::min<int64_t>((nnode + 255) / 256, 1 << 16);
-  reset_nodes<<<std::max(nb, 1u), 256, 0, s>>>(w.nd, nnode); count_launch();
-  // the forest's saddles are the live list of the exact rounds
-  return run_rounds_from(w, T, w.forest, forest_n, w.live0, w.ctr + 0, s, dstatus);
+  return DMS_OK;
+}
+
+// pairs the live saddles in w.live0 (ctr[kCtrLive], of nsad) over nnode nodes:
+// Borůvka rounds collect the spanning forest's saddles, the exact rounds pair
+// them (forest false: the exact rounds on all live saddles)
+int run_pairing(DiagWs& w, Tri T, int64_t nsad, int64_t nnode, cudaStream_t s, int32_t* dstatus,
+                bool forest) {
+  Rounds r;
+  r.T = T;
+  r.nd = w.nd;
+  r.cur = w.live0;
+  r.nxt = forest ? w.live1 : w.forest;
+  r.n = w.ctr + kCtrLive;
+  r.round = 1;
+  r.forest = forest ? w.forest : nullptr;
+  r.forest_only = false;
+  r.first_found = forest;
+  r.left = w.live1;
+  r.ctr = w.ctr;
+  r.n_dev = nullptr;
+  r.nnode = nnode;
+  if (nsad > kOneLaunch) {
+    uint32_t *cur = r.cur, *nxt = r.nxt;
+    unsigned int *cur_n = w.ctr + kCtrLive, *nxt_n = w.ctr + kCtrNext, h = 0;
+    DMS_CUDA_OK(cudaMemcpyAsync(&h, cur_n, sizeof(h), cudaMemcpyDeviceToHost, s));
+    DMS_CUDA_OK(cudaStreamSynchronize(s));
+    if (forest) {
+      const bool more = (int64_t)h > kOneLaunch;
+      DMS_TRY(run_large(w, T, cur, cur_n, nxt, nxt_n, r.round, h, true, true, s));
+      r.cur = cur;
+      r.nxt = nxt;
+      r.n = cur_n;
+      r.forest_only = true;
+      r.first_found = !more;
+      DMS_TRY(launch_rounds(r, kOneLaunch, dstatus, s));
+      const unsigned int nb = (unsigned int)std::min<int64_t>((nnode + 255) / 256, 1 << 16);
+      reset_nodes<<<std::max(nb, 1u), 256, 0, s>>>(w.nd, nullptr, nnode); count_launch();
+      DMS_CUDA_OK(cudaMemcpyAsync(&h, w.ctr + kCtrForest, sizeof(h), cudaMemcpyDeviceToHost, s));
+      DMS_CUDA_OK(cudaMemsetAsync(w.ctr + kCtrRound, 0, (kCtrWords - kCtrRound) * sizeof(unsigned int), s));
+      DMS_CUDA_OK(cudaStreamSynchronize(s));
+      cur = w.forest;
+      cur_n = w.ctr + kCtrForest;
+      nxt = w.live0;
+      nxt_n = w.ctr + kCtrLive;
+      r.round = 1;
+      r.forest = nullptr;
+      r.forest_only = r.first_found = false;
+    }
+    DMS_TRY(run_large(w, T, cur, cur_n, nxt, nxt_n, r.round, h, false, false, s));
+    r.cur = cur;
+    r.nxt = nxt;
+    r.n = cur_n;
+  }
+  DMS_TRY(launch_rounds(r, nsad, dstatus, s));
+  return finish_sorted(w, T, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1191,8 +1450,8 @@ __global__ void sc_result(const uint32_t* __restrict__ live, const unsigned int*
 constexpr int kMaxSelfCorrectingRounds = 1 << 16;
 
 int run_selfcorrecting(DiagWs& w, Tri T, int64_t nnode, cudaStream_t s, int32_t* dstatus) {
-  unsigned int* live_n = w.ctr + 0;
-  unsigned int* changed = w.ctr + 3;
+  unsigned int* live_n = w.ctr + kCtrLive;
+  unsigned int* changed = w.ctr + kCtrChanged;
   unsigned int h = 0;
   DMS_CUDA_OK(cudaMemcpyAsync(&h, live_n, sizeof(h), cudaMemcpyDeviceToHost, s));
   DMS_CUDA_OK(cudaStreamSynchronize(s));
@@ -1256,7 +1515,7 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
   auto nb = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, (n + TB - 1) / TB); };
 
   // ---- D0
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   if (nc[0] > 0) {
     init_nodes_d0<<<nb(nc[0]), TB, 0, s>>>(order, crit0, nc[0], w.nd); count_launch();
     write_essential<<<nb(nc[0]), TB, 0, s>>>(f, order, crit0, nc[0], ess); count_launch();
@@ -1266,20 +1525,20 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
     mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.claim); count_launch();
     d0_weights<<<nb(nc[1]), TB, 0, s>>>(D, order, crit1, nc[1], w.T0); count_launch();
     const DescWalk<OneField> wk{OneField{g}, crit1, desc, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, nc[1], w.ctr + 6, w.T0, dstatus, s));
+    DMS_TRY(launch_walks(wk, nullptr, nc[1], w.ctr + kCtrWalk, w.T0, dstatus, s));
     w.nd.immortal = kNone;  // every minimum but the global one can die
-    link_walks<<<nb(nc[1]), TB, 0, s>>>(nc[1], w.T0, w.live0, w.ctr + 0, dstatus, false,
+    link_walks<<<nb(nc[1]), TB, 0, s>>>(nc[1], w.T0, w.live0, w.ctr + kCtrLive, dstatus, false,
                                         pairing == 0, w.nd); count_launch();
   }
   w.nd.immortal = kNone;
   int st = pairing == 1 ? run_selfcorrecting(w, w.T0, std::max<int64_t>(nc[0], 1), s, dstatus)
-                        : run_pairing(w, w.T0, std::max<int64_t>(nc[0], 1), s, dstatus, true);
+                        : run_pairing(w, w.T0, nc[1], std::max<int64_t>(nc[0], 1), s, dstatus, true);
   if (st) return st;
   st = write_diagram(0, w, D, f, order, crit0, crit1, nc[1], d0, cap0, n_out + 0, dstatus, s);
   if (st) return st;
 
   // ---- D2
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   init_nodes_d2<<<nb(nc[3] + 1), TB, 0, s>>>(D, order, crit3, nc[3], w.nd); count_launch();
   if (nc[2] > 0) {
     DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, w.nclaim * sizeof(uint32_t), s));
@@ -1288,14 +1547,14 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
     }
     d2_weights<<<nb(nc[2]), TB, 0, s>>>(D, order, crit2, nc[2], w.T2); count_launch();
     const DualWalk<OneField> wk{OneField{g}, crit2, rec, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, nc[2], w.ctr + 6, w.T2, dstatus, s));
+    DMS_TRY(launch_walks(wk, nullptr, nc[2], w.ctr + kCtrWalk, w.T2, dstatus, s));
     w.nd.immortal = 0;  // OUTSIDE
-    link_walks<<<nb(nc[2]), TB, 0, s>>>(nc[2], w.T2, w.live0, w.ctr + 0, dstatus, false,
+    link_walks<<<nb(nc[2]), TB, 0, s>>>(nc[2], w.T2, w.live0, w.ctr + kCtrLive, dstatus, false,
                                         pairing == 0, w.nd); count_launch();
   }
   w.nd.immortal = 0;
   st = pairing == 1 ? run_selfcorrecting(w, w.T2, nc[3] + 1, s, dstatus)
-                    : run_pairing(w, w.T2, nc[3] + 1, s, dstatus, true);
+                    : run_pairing(w, w.T2, nc[2], nc[3] + 1, s, dstatus, true);
   if (st) return st;
   st = write_diagram(2, w, D, f, order, crit2, crit3, nc[2], d2, cap2, n_out + 1, dstatus, s);
   if (st) return st;
@@ -1486,23 +1745,6 @@ __global__ void b_d2_weights(const FieldTab ft, const uint32_t* __restrict__ ord
     T.s[i].res = kNone;
     T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
   }
-}
-
-// node arrays back to singletons between the forest and the pairing rounds
-// (node count on the device)
-__global__ void b_reset_nodes(Nodes nd, const int64_t* __restrict__ cnt, int64_t extra) {
-  const int64_t n = *cnt + extra;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    nd.parent[i] = (uint32_t)i;
-    nd.best[i] = 0ull;
-  }
-}
-
-// the fixed number of Borůvka rounds must have emptied the live list (they
-// do: active components at least halve per round)
-__global__ void b_forest_done(const unsigned int* __restrict__ live_n, int32_t* dstatus) {
-  if (threadIdx.x == 0 && blockIdx.x == 0 && *live_n != 0) set_status(dstatus, DMS_ERR_TIMEOUT);
 }
 
 // As link_walks with tag set: also the forest's first round search (both
@@ -1703,9 +1945,8 @@ __global__ void __launch_bounds__(PNT) b_write_pairs(int dim, const FieldTab ft,
 
 }  // namespace
 
-constexpr int kBatchRounds = 96;
-constexpr int kBoruvkaRounds = 40;
-int diagram_batch_rounds() { return kBatchRounds; }
+constexpr unsigned int kBatchLarge = 6;  // (live saddles fall to a third per round or faster)
+int diagram_batch_rounds() { return (int)kMaxExactRounds; }
 
 // Workspace of the batched pairing: the DiagWs of the capacities plus the
 // per-field counters and pair-tile sums.
@@ -1741,48 +1982,76 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   const unsigned G = (unsigned)sms * 8, TB = 256;  // grid-stride launches
   DMS_CUDA_OK(cudaMemsetAsync(fcount, 0, 2 * (nfields + 1) * sizeof(unsigned long long), s));
 
-  bool mem_ok = true;
-  // the spanning forest by Borůvka rounds, then the exact rounds on its
-  // saddles (as in the single-field path), all with fixed round counts
-  auto rounds = [&](Tri T, const int64_t* ncnt, int64_t extra) {
-    uint32_t* cur = w.live0;
-    uint32_t* nxt = w.live1;
-    unsigned int* cur_n = w.ctr + 0;
-    unsigned int* nxt_n = w.ctr + 1;
-    unsigned int* forest_n = w.ctr + 2;
-    mem_ok = mem_ok && cudaMemsetAsync(forest_n, 0, sizeof(unsigned int), s) == cudaSuccess;
-    for (int r = 1; r <= kBoruvkaRounds; ++r) {
+  // the spanning forest and the exact rounds on its saddles, as in the
+  // single-field path, the node count (ncnt + extra) read on the device
+  const bool large = nsad > kOneLaunch;
+  auto rounds = [&](Tri T, const int64_t* ncnt, int64_t extra) -> int {
+    // kBatchLarge rounds of one launch per phase (they do nothing on an empty
+    // list), the rest in one launch
+    uint32_t *cur = w.live0, *nxt = w.live1;
+    unsigned int *cur_n = w.ctr + kCtrLive, *nxt_n = w.ctr + kCtrNext;
+    bool mem_ok = true;
+    unsigned int round = 1;
+    for (; large && round <= kBatchLarge; ++round) {
       mem_ok = mem_ok && cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s) == cudaSuccess;
-      if (r > 1) {  // b_link_walks did round 1's search
-        round_find<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, (uint64_t)r); count_launch();
+      if (round > 1) {  // b_link_walks did round 1's search
+        round_find<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round); count_launch();
       }
-      boruvka_hook<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, (uint64_t)r, nxt, nxt_n, w.forest,
-                                    forest_n); count_launch();
+      boruvka_hook<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n, w.forest,
+                                    w.ctr + kCtrForest); count_launch();
       std::swap(cur, nxt);
       std::swap(cur_n, nxt_n);
     }
-    b_forest_done<<<1, 32, 0, s>>>(cur_n, dstatus); count_launch();
-    b_reset_nodes<<<G, TB, 0, s>>>(w.nd, ncnt, extra); count_launch();
-    cur = w.forest;
-    cur_n = forest_n;
-    nxt = w.live0;
-    nxt_n = w.ctr + 0;
-    for (int r = 1; r <= kBatchRounds; ++r) {
-      mem_ok = mem_ok && cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s) == cudaSuccess;
-      round_find<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, (uint64_t)r); count_launch();
-      round_merge<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, (uint64_t)r, nxt, nxt_n); count_launch();
-      std::swap(cur, nxt);
-      std::swap(cur_n, nxt_n);
+    Rounds r;
+    r.T = T;
+    r.nd = w.nd;
+    r.cur = cur;
+    r.nxt = nxt;
+    r.n = cur_n;
+    r.round = round;
+    r.forest = w.forest;
+    r.forest_only = large;
+    r.first_found = round == 1;
+    r.left = w.live1;
+    r.ctr = w.ctr;
+    r.n_dev = ncnt;
+    r.nnode = extra;
+    DMS_TRY(launch_rounds(r, nsad, dstatus, s));
+    if (large) {
+      reset_nodes<<<G, TB, 0, s>>>(w.nd, ncnt, extra); count_launch();
+      mem_ok = mem_ok && cudaMemsetAsync(w.ctr + kCtrRound, 0, (kCtrWords - kCtrRound) * sizeof(unsigned int),
+                                         s) == cudaSuccess;
+      cur = w.forest;
+      cur_n = w.ctr + kCtrForest;
+      nxt = w.live0;
+      nxt_n = w.ctr + kCtrLive;
+      for (round = 1; round <= kBatchLarge; ++round) {
+        mem_ok = mem_ok && cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s) == cudaSuccess;
+        round_find<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round); count_launch();
+        round_merge<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n); count_launch();
+        std::swap(cur, nxt);
+        std::swap(cur_n, nxt_n);
+      }
+      r.cur = cur;
+      r.nxt = nxt;
+      r.n = cur_n;
+      r.round = round;
+      r.forest = nullptr;
+      r.forest_only = r.first_found = false;
+      DMS_TRY(launch_rounds(r, nsad, dstatus, s));
     }
-    b_finish<<<1, 1024, 0, s>>>(cur, cur_n, T, w.nd, dstatus); count_launch();
+    if (!mem_ok) return DMS_ERR_CUDA;
+    const unsigned int* left_n = w.ctr + kCtrLeft;
+    b_finish<<<1, 1024, 0, s>>>(w.live1, left_n, T, w.nd, dstatus); count_launch();
     // more than the one-CTA finish holds: sort them by weight on the device
     // and finish them in that order (one thread; nothing runs when the
     // count is small)
-    unsigned int* big_n = w.ctr + 4;
-    b_big_count<<<1, 32, 0, s>>>(cur_n, big_n); count_launch();
-    gather_live<<<G, TB, 0, s>>>(cur, big_n, T, w.rb.ka, w.rb.va); count_launch();
+    unsigned int* big_n = w.ctr + kCtrBig;
+    b_big_count<<<1, 32, 0, s>>>(left_n, big_n); count_launch();
+    gather_live<<<G, TB, 0, s>>>(w.live1, big_n, T, w.rb.ka, w.rb.va); count_launch();
     const bool in_a = radix64::sort(w.rb, nsad, 44, s, big_n);
     sequential_finish<<<1, 32, 0, s>>>(in_a ? w.rb.va : w.rb.vb, big_n, T, w.nd); count_launch();
+    return DMS_OK;
   };
   auto write = [&](int dim, Tri T, const int64_t* critA, const int64_t* critB, const int64_t* n_dev,
                    dms_pair* out, int64_t* offs, int64_t* total, unsigned long long* fc) {
@@ -1795,7 +2064,7 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   };
 
   // ---- D0
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   b_init_nodes_d0<<<G, TB, 0, s>>>(order, crit[0], cnt_dev, w.nd); count_launch();
   b_essential<<<G, TB, 0, s>>>(ft, f, order, crit[0], cnt_dev, ess); count_launch();
   DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, total_vertices * sizeof(uint32_t), s));
@@ -1803,29 +2072,28 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   b_d0_weights<<<G, TB, 0, s>>>(ft, order, crit[1], cnt_dev, w.T0); count_launch();
   {
     const DescWalk<ManyFields> wk{ManyFields{fields_dev, nfields}, crit[1], desc, w.claim};
-    DMS_TRY(launch_walks(wk, cnt_dev + 1, 0, w.ctr + 6, w.T0, dstatus, s));
+    DMS_TRY(launch_walks(wk, cnt_dev + 1, 0, w.ctr + kCtrWalk, w.T0, dstatus, s));
   }
   w.nd.immortal = kNone;
-  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 1, w.T0, w.live0, w.ctr + 0, dstatus, w.nd); count_launch();
-  rounds(w.T0, cnt_dev + 0, 0);
+  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 1, w.T0, w.live0, w.ctr + kCtrLive, dstatus, w.nd); count_launch();
+  DMS_TRY(rounds(w.T0, cnt_dev + 0, 0));
   write(0, w.T0, crit[0], crit[1], cnt_dev + 1, d0, pair_offsets, pair_totals + 0, fcount);
 
   // ---- D2
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   b_init_nodes_d2<<<G, TB, 0, s>>>(ft, order, crit[3], cnt_dev, w.nd); count_launch();
   DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, w.nclaim * sizeof(uint32_t), s));
   mark_ends<<<G, TB, 0, s>>>(crit[3], cnt_dev + 3, 0, 1, w.claim); count_launch();
   b_d2_weights<<<G, TB, 0, s>>>(ft, order, crit[2], cnt_dev, w.T2); count_launch();
   {
     const DualWalk<ManyFields> wk{ManyFields{fields_dev, nfields}, crit[2], rec, w.claim};
-    DMS_TRY(launch_walks(wk, cnt_dev + 2, 0, w.ctr + 6, w.T2, dstatus, s));
+    DMS_TRY(launch_walks(wk, cnt_dev + 2, 0, w.ctr + kCtrWalk, w.T2, dstatus, s));
   }
   w.nd.immortal = 0;  // OUTSIDE, shared by all fields
-  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 2, w.T2, w.live0, w.ctr + 0, dstatus, w.nd); count_launch();
-  rounds(w.T2, cnt_dev + 3, 1);
+  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 2, w.T2, w.live0, w.ctr + kCtrLive, dstatus, w.nd); count_launch();
+  DMS_TRY(rounds(w.T2, cnt_dev + 3, 1));
   write(2, w.T2, crit[2], crit[3], cnt_dev + 2, d2, pair_offsets + (nfields + 1), pair_totals + 1,
         fcount + (nfields + 1));
-  if (!mem_ok) return DMS_ERR_CUDA;
   return launch_status();
 }
 
@@ -2188,7 +2456,7 @@ int launch_diagram2d(const float* f, const uint32_t* order, const uint8_t* desc,
   };
 
   // ---- D0
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   init_nodes_d0<<<nb(nc[0]), TB, 0, s>>>(order, crit0, nc[0], w.nd); count_launch();
   write_essential<<<nb(nc[0]), TB, 0, s>>>(f, order, crit0, nc[0], ess); count_launch();
   if (ne > 0) {
@@ -2196,17 +2464,17 @@ int launch_diagram2d(const float* f, const uint32_t* order, const uint8_t* desc,
     mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.claim); count_launch();
     d0_weights2d<<<nb(ne), TB, 0, s>>>(g, order, crit1, ne, w.T0); count_launch();
     const DescWalk2d wk{g, crit1, desc, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + 6, w.T0, dstatus, s));
-    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + 0, dstatus); count_launch();
+    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + kCtrWalk, w.T0, dstatus, s));
+    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + kCtrLive, dstatus); count_launch();
   }
   w.nd.immortal = kNone;
-  int st = run_rounds(w, w.T0, s, dstatus);
+  int st = run_pairing(w, w.T0, ne, nc[0], s, dstatus, false);
   if (st) return st;
   st = write(0, crit0, d0, cap0, n_out + 0);
   if (st) return st;
 
   // ---- D1
-  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(unsigned int), s));
+  DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   init_nodes_d1_2d<<<nb(nc[2] + 1), TB, 0, s>>>(g, order, crit2, nc[2], w.nd); count_launch();
   if (ne > 0) {
     DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, 2 * g.n * sizeof(uint32_t), s));
@@ -2215,11 +2483,11 @@ int launch_diagram2d(const float* f, const uint32_t* order, const uint8_t* desc,
     }
     d1_weights2d<<<nb(ne), TB, 0, s>>>(g, order, crit1, ne, w.T0); count_launch();
     const DualWalk2d wk{g, crit1, rec, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + 6, w.T0, dstatus, s));
-    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + 0, dstatus, true); count_launch();
+    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + kCtrWalk, w.T0, dstatus, s));
+    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + kCtrLive, dstatus, true); count_launch();
   }
   w.nd.immortal = 0;  // OUTSIDE
-  st = run_rounds(w, w.T0, s, dstatus);
+  st = run_pairing(w, w.T0, ne, nc[2] + 1, s, dstatus, false);
   if (st) return st;
   st = write(1, crit2, d1, cap1, n_out + 1);
   if (st) return st;
