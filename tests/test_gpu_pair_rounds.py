@@ -14,9 +14,11 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
+import oracle
+import oracle_jobs
 import paper_2505_21266_gb300 as dms
 from paper_2505_21266_gb300 import fields
-from test_gpu_configs import chain_field
+from test_gpu_configs import _same_pairs, chain_field
 
 
 def _same(f):
@@ -41,3 +43,16 @@ def test_rounds_by_size(shape, lo, hi):
 @pytest.mark.parametrize("n", [60, 70, 4090, 4100, 9000])
 def test_chain_of_wells(n):
     _same(torch.from_numpy(np.ascontiguousarray(chain_field(n))).cuda())
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 1026, 32 * 1024 + 1, 33 * 1024 + 2])
+def test_pair_lists_at_tile_edges(n):
+    """n - 1 saddles, all paired: the pair writer's tiles of 1024 full, one
+    short and one over, and more tiles than one warp looks back over at once."""
+    f_np = np.ascontiguousarray(chain_field(n, deeper_right=False))
+    r = oracle.run(f_np)
+    res = dms.diagram(torch.from_numpy(f_np).cuda())
+    assert int(res.crit[1].numel()) == n - 1
+    d0, d2, _ = oracle_jobs.sorted_pairs(r)
+    _same_pairs(res.diagrams.numpy("d0"), d0)
+    _same_pairs(res.diagrams.numpy("d2"), d2)
