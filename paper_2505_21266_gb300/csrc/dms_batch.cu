@@ -32,8 +32,8 @@ int launch_critical(const uint8_t* desc, const uint64_t* rec, const Grid& g, int
 size_t diagram_batch_workspace_bytes(int64_t nfields, const int64_t* caps, int64_t total);
 int diagram_batch_rounds();
 int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* desc,
-                         const uint64_t* rec, const dms_field_desc* fields_dev, int nfields,
-                         int64_t total_vertices, int64_t* const crit[4], const int64_t* cnt_dev,
+                         const uint64_t* rec, const dms_field_desc* fields_host,
+                         const dms_field_desc* fields_dev, int nfields, int64_t total_vertices, int64_t* const crit[4], const int64_t* cnt_dev,
                          const int64_t* caps, dms_pair* d0, dms_pair* d2, int64_t cap_pairs,
                          int64_t* pair_offsets, dms_pair* ess, int64_t* pair_totals, void* ws,
                          int32_t* dstatus, cudaStream_t s);
@@ -189,7 +189,7 @@ int dms_batch_diagrams(const float* f, const dms_field_desc* fields_host,
                             w.crit_ws, dstatus, s);
   if (st) return st;
   dms::clamp_counts_kernel<<<1, 32, 0, s>>>(counts, caps[0], caps[1], caps[2], caps[3], w.eff); dms::count_launch();
-  return dms::launch_diagram_batch(f, order, desc, rec, fields_dev, nfields, total, w.crit, w.eff,
+  return dms::launch_diagram_batch(f, order, desc, rec, fields_host, fields_dev, nfields, total, w.crit, w.eff,
                                    caps, d0, d2, cap_pairs, pair_offsets, d0_essential, counts + 4,
                                    w.diag_ws, dstatus, s);
 }

@@ -95,6 +95,13 @@ __device__ __forceinline__ void xyz(const Grid& g, int64_t v, int64_t& x, int64_
   y = yy;
   x = r - yy * nx;
 }
+__device__ __forceinline__ void coords(const Grid& g, int64_t v, int& x, int& y, int& z) {
+  int64_t x64, y64, z64;
+  xyz(g, v, x64, y64, z64);
+  x = (int)x64;
+  y = (int)y64;
+  z = (int)z64;
+}
 // is anchor + corner c inside the grid, for c in {0..7} with all of +c
 __device__ __forceinline__ bool fits(const Grid& g, int64_t ax, int64_t ay, int64_t az, int c) {
   return ax >= 0 && ay >= 0 && az >= 0 && ax + (c & 1) < g.nx && ay + ((c >> 1) & 1) < g.ny &&
@@ -118,25 +125,6 @@ __device__ __forceinline__ uint32_t local_rank(const Dev& D, const uint32_t* __r
   return r;
 }
 
-// ranks of two lower neighbours u1, u2 of t among its lower neighbours
-__device__ __forceinline__ void local_rank2(const Dev& D, const uint32_t* __restrict__ order,
-                                           int64_t t, uint32_t o1, uint32_t o2, uint32_t& r1,
-                                           uint32_t& r2) {
-  int64_t x, y, z;
-  xyz(D.g, t, x, y, z);
-  r1 = r2 = 0;
-#pragma unroll
-  for (int s = 0; s < 14; ++s) {
-    int c = cSlotCorner[s];
-    int sg = s < 7 ? 1 : -1;
-    int64_t nx = x + sg * (c & 1), ny = y + sg * ((c >> 1) & 1), nz = z + sg * ((c >> 2) & 1);
-    if (nx < 0 || ny < 0 || nz < 0 || nx >= D.g.nx || ny >= D.g.ny || nz >= D.g.nz) continue;
-    const uint32_t on = __ldg(order + t + D.slot_delta[s]);
-    r1 += on < o1 ? 1u : 0u;
-    r2 += on < o2 ? 1u : 0u;
-  }
-}
-
 // tet type of the chain 0 < c1 < c2 < 7 (c1 one corner bit, c2 two): the
 // types are ordered by c1, then by whether the bit c2 adds is the larger of
 // the two bits c1 leaves
@@ -152,9 +140,8 @@ __device__ __forceinline__ int tet_type(int c1, int c2) {
 //  * code 4 omits the top: anchored at anchor - (7 ^ c2), chain
 //    (7 ^ c2, (7 ^ c2) | c1);
 //  * code 2 / 3 omit c1 / c2: same anchor, chain (c2 ^ c1, c2) / (c1, c1 | (7 ^ c2)).
-// Entry 4k + code - 1 is a byte: next type (bits 0-2), anchor step corner
-// (3-5), step sign (6-7: 0 none, 1 plus, 2 minus); 24 entries in three
-// 64-bit immediates.
+// entry(4k + code - 1): next type (bits 0-2), anchor step corner (3-5), step
+// sign (6-7: 0 none, 1 plus, 2 minus).
 namespace dual_step_detail {
 constexpr int c1_of(int k) { return (0x442211 >> (4 * k)) & 15; }
 constexpr int c2_of(int k) { return (0x656353 >> (4 * k)) & 15; }
@@ -168,55 +155,42 @@ constexpr uint64_t entry(int e) {
   else { n1 = c1; n2 = c1 | (7 ^ c2); }
   return (uint64_t)(type_of(n1, n2) | (stp << 3) | (sg << 6));
 }
-constexpr uint64_t word(int w) {
-  uint64_t x = 0;
-  for (int i = 0; i < 8; ++i) x |= entry(8 * w + i) << (8 * i);
-  return x;
-}
 }  // namespace dual_step_detail
-constexpr uint64_t kDualStep0 = dual_step_detail::word(0);
-constexpr uint64_t kDualStep1 = dual_step_detail::word(1);
-constexpr uint64_t kDualStep2 = dual_step_detail::word(2);
-__device__ __forceinline__ uint32_t dual_step(int k, uint32_t code) {
-  const uint32_t e = 4 * k + code - 1;
-  const uint64_t w = e < 8 ? kDualStep0 : (e < 16 ? kDualStep1 : kDualStep2);
-  return (uint32_t)(w >> (8 * (e & 7))) & 255u;
-}
-
-// Walks with path sharing: every vertex (D0) or non-critical tet (D2) a walk
-// passes is claimed for it (atomicCAS on claim[id]); a walk that reaches an id
-// claimed by another walk stops there, since from there on both follow the
-// same path, and records kLinkBit | that walk instead of an end node.
-constexpr uint32_t kLinkBit = 0x80000000u;
-constexpr uint32_t kUnclaimed = 0xFFFFFFFFu;
-
-// Before the walks, every end (minimum, critical tet) holds an end mark,
-// kLinkBit | its node, in its claim word; a walk's claim fails there and the
-// walk ends with that node, without a search of the critical list.  A
-// claim word thus holds a walk id (a walk passed) or an end mark, and a walk
-// that fails a claim records old ^ kLinkBit: a link to that walk, or the node.
-__device__ __forceinline__ uint32_t claim_result(uint32_t old) { return old ^ kLinkBit; }
+// ---------------------------------------------------------------------------
+// v-paths by bricks.
+//
+// A path (vertex -> paired edge -> other vertex; tet -> paired facet -> other
+// cofacet) is followed cell by cell only inside bricks of up to 8192 cells, in
+// shared memory, for all cells of a brick at once: every cell then knows where
+// its path ends or leaves the brick, and a walk hops from brick to brick.
+// Every cell has one word:
+//   bit 31 set    the end: bits 0..30 the node (0 for OUTSIDE in the dual)
+//   bit 31 clear  where the path goes on: bits 13..18 the brick (two bits per
+//                 axis: 0, 1, 2 for the one before, this one, the next), bits
+//                 0..12 the cell in it
+// mark_ends gives the cells at path ends (minima, critical tets) their nodes
+// first; resolve_paths reads them there.
+// Followed cell by cell through memory, one load and one claim by
+// compare-and-swap per step, a walk was a chain of 3 (vertices) and 10 (tets)
+// dependent steps on average on noise, up to 400 on smooth fields, 1 us each;
+// hops are 1.3 to 2.7 on average, up to 27.  Resolving all cells costs about
+// 100 instructions per tet and a word per cell written, which noise, whose
+// paths are short, pays back in fewer random reads: D0/D2 stage 64^3 mixture
+// 705 -> 356 us, 128^3 smooth 953 -> 368 us, 16384^2 37.8 -> 30.8 ms, 512^3
+// ties 28.9 -> 25.5 ms, 1024^3 87.7 -> 76.6 ms.  Following every cell to its
+// end in turn instead of doubling took 147 ms there.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kEnd = 0x80000000u;
+constexpr uint32_t kNoMark = kEnd | 0x7FFFFFFFu;  // an end without a node, or bad data
+constexpr uint32_t kLoop = kEnd | 0x7FFFFFFEu;    // a path that does not end (bad data)
+constexpr uint32_t kFinal = 0x40000000u;          // (in shared memory) a way on, out of the brick
 
 __global__ void mark_ends(const int64_t* __restrict__ list, const int64_t* n_dev, int64_t n_host,
-                          uint32_t node0, uint32_t* claim) {
+                          uint32_t node0, uint32_t* path) {
   const int64_t n = n_dev ? *n_dev : n_host;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    claim[list[i]] = kLinkBit | (uint32_t)(i + node0);
-}
-
-// the node a walk ends at, following the walks it joined
-__device__ __forceinline__ uint32_t resolve_walk(const Sad* __restrict__ sd, uint32_t x,
-                                                 int64_t nwalks, int32_t* dstatus) {
-  for (int64_t it = 0; (x & kLinkBit) && it <= nwalks; ++it) {
-    const uint32_t w = x & ~kLinkBit;
-    x = (w & 1) ? sd[w >> 1].rb : sd[w >> 1].ra;
-  }
-  if (x & kLinkBit) {
-    set_status(dstatus, DMS_ERR_TIMEOUT);
-    return 0;
-  }
-  return x;
+    path[list[i]] = kEnd | (uint32_t)(i + node0);
 }
 
 // Appends of a whole CTA (256 threads) to two lists at once: one atomic per
@@ -255,23 +229,6 @@ __device__ __forceinline__ void cta_append2(CtaAppend& sh, bool w0, uint32_t* l0
 }
 
 
-// D0: the weight of each critical edge (its lexicographic key).
-__global__ void d0_weights(Dev D, const uint32_t* __restrict__ order,
-                           const int64_t* __restrict__ crit1, int64_t ne, Tri T) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= ne) return;
-  int64_t id = crit1[i];
-  int64_t a = id / 7;
-  int k = (int)(id - a * 7);
-  int64_t b = a + corner_delta(D.g, edge_corner(k));
-  uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
-  int64_t top = oa > ob ? a : b;
-  uint32_t r = local_rank(D, order, top, oa > ob ? ob : oa);
-  T.s[i].w = ((uint64_t)(oa > ob ? oa : ob) << 4) | r;
-  T.s[i].res = kNone;
-  T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
-}
-
 // The two cofacets of critical triangle id (anchor a, type k) in field g
 // (anchor coordinates ax, ay, az); -1 where a cofacet leaves the grid.
 __device__ __forceinline__ void tri_cofacets(const Grid& g, int64_t a, int k, int64_t ax,
@@ -298,40 +255,6 @@ __device__ __forceinline__ void tri_cofacets(const Grid& g, int64_t a, int k, in
   }
 }
 
-// D2: the weight of each critical triangle (decreasing triangle key).
-__global__ void d2_weights(Dev D, const uint32_t* __restrict__ order,
-                           const int64_t* __restrict__ crit2, int64_t nt, Tri T) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= nt) return;
-  int64_t id = crit2[i];
-  int64_t a = id / 12;
-  int k = (int)(id - a * 12);
-  const int p = tri_p(k), q = tri_q(k);
-  int64_t v[3] = {a, a + corner_delta(D.g, p), a + corner_delta(D.g, q)};
-  uint32_t o[3] = {__ldg(order + v[0]), __ldg(order + v[1]), __ldg(order + v[2])};
-  int it = 0;
-  if (o[1] > o[it]) it = 1;
-  if (o[2] > o[it]) it = 2;
-  uint32_t om = 0, ol = 0xFFFFFFFFu;
-  for (int j = 0; j < 3; ++j)
-    if (j != it) {
-      om = max(om, o[j]);
-      ol = min(ol, o[j]);
-    }
-  uint32_t rm, rl;
-  local_rank2(D, order, v[it], om, ol, rm, rl);
-  uint64_t key = ((uint64_t)o[it] << 8) | (rm << 4) | rl;
-  T.s[i].w = kMask44 - key;
-  T.s[i].res = kNone;
-  T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
-}
-
-// ---------------------------------------------------------------------------
-// v-path walks.  Each saddle owns two walks (2s and 2s + 1); a walk's result
-// (its end node, or kLinkBit | the walk it joined) goes to T.ra / T.rb.  A
-// walk policy gives the start of a walk and one step of it.
-// ---------------------------------------------------------------------------
-
 // one field for the whole call
 struct OneField {
   Grid g;
@@ -339,24 +262,25 @@ struct OneField {
     out = g;
     off = 0;
   }
-  __device__ __forceinline__ void coords(const Grid&, int64_t v, int64_t& x, int64_t& y,
-                                         int64_t& z) const {
-    xyz(g, v, x, y, z);
+  // brick id of 2^lx x 2^ly x 2^lz vertices: its field, its place in it
+  __device__ __forceinline__ void brick(int64_t id, int lx, int ly, int lz, Grid& out, int64_t& off,
+                                        int& bx, int& by, int& bz) const {
+    get(0, out, off);
+    const uint32_t tx = (uint32_t)((g.nx + (1 << lx) - 1) >> lx), ty = (uint32_t)((g.ny + (1 << ly) - 1) >> ly);
+    const uint32_t i = (uint32_t)id, r = i / tx;
+    bx = (int)(i - r * tx);
+    bz = (int)(r / ty);
+    by = (int)(r - (uint32_t)bz * ty);
+    (void)lz;
   }
 };
 
-// a batch: the field that holds an anchor, by binary search of the table
+// a batch: the field that holds an anchor or a brick, by binary search
 struct ManyFields {
   const dms_field_desc* fd;
   int n;
-  __device__ __forceinline__ void get(int64_t anchor, Grid& out, int64_t& off) const {
-    int lo = 0, hi = n;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (fd[mid].offset <= anchor) lo = mid;
-      else hi = mid;
-    }
-    const dms_field_desc d = fd[lo];
+  const int64_t* brick0;  // nfields + 1: the fields' first bricks (see brick_table)
+  __device__ __forceinline__ void set(const dms_field_desc& d, Grid& out, int64_t& off) const {
     out.nx = d.nx;
     out.ny = d.ny;
     out.nz = d.nz;
@@ -364,9 +288,26 @@ struct ManyFields {
     out.n = out.sxy * d.nz;
     off = d.offset;
   }
-  __device__ __forceinline__ void coords(const Grid& g, int64_t v, int64_t& x, int64_t& y,
-                                         int64_t& z) const {
-    xyz(g, v, x, y, z);
+  __device__ __forceinline__ void get(int64_t anchor, Grid& out, int64_t& off) const {
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (fd[mid].offset <= anchor) lo = mid;
+      else hi = mid;
+    }
+    set(fd[lo], out, off);
+  }
+  __device__ __forceinline__ void brick(int64_t id, int lx, int ly, int lz, Grid& out, int64_t& off,
+                                        int& bx, int& by, int& bz) const {
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (__ldg(brick0 + mid) <= id) lo = mid;
+      else hi = mid;
+    }
+    set(fd[lo], out, off);
+    OneField{out}.brick(id - __ldg(brick0 + lo), lx, ly, lz, out, off, bx, by, bz);
+    off = fd[lo].offset;
   }
 };
 
@@ -376,271 +317,385 @@ __device__ __forceinline__ int64_t slot_delta_g(const Grid& g, int s) {
   return s < 7 ? d : -d;
 }
 
-// D0: descending paths from the two vertices of a critical edge to minima
+// A cell of a brick: its vertex's coordinates in one word, eight bits per
+// axis, each offset by the brick's extent, so that after a step the bits above
+// the coordinate's say which brick it is in: 0, 1 (this one) or 2.
+template <class P>
+__device__ __forceinline__ uint32_t packed_coords(int lv) {
+  return ((lv & ((1 << P::LX) - 1)) + (1 << P::LX)) |
+         (((lv >> P::LX) & ((1 << P::LY) - 1)) + (1 << P::LY)) << 8 |
+         ((lv >> (P::LX + P::LY)) + (1 << P::LZ)) << 16;
+}
+__device__ __forceinline__ constexpr uint32_t packed_step(int dx, int dy, int dz) {
+  return (uint32_t)(dx + dy * 256 + dz * 65536);
+}
+// cell k of the vertex at c as a word: a cell of the brick, or a way out of it
+template <class P>
+__device__ __forceinline__ uint32_t brick_word(uint32_t c, int k) {
+  const uint32_t lv = (c & ((1u << P::LX) - 1)) | (c >> 8 & ((1u << P::LY) - 1)) << P::LX |
+                      (c >> 16 & ((1u << P::LZ) - 1)) << (P::LX + P::LY);
+  const uint32_t dir = (c >> P::LX & 3u) | (c >> (8 + P::LY) & 3u) << 2 | (c >> (16 + P::LZ) & 3u) << 4;
+  const uint32_t local = lv * P::K + k;
+  return dir == 21u ? local : kFinal | dir << 13 | local;
+}
+// is the vertex at c inside [0, mx) x [0, my) x [0, mz) of the brick at (x0, y0, z0)
+template <class P>
+__device__ __forceinline__ bool inside(uint32_t c, int x0, int y0, int z0, uint32_t mx, uint32_t my,
+                                       uint32_t mz) {
+  return (uint32_t)(x0 + (int)(c & 255u) - (1 << P::LX)) < mx &&
+         (uint32_t)(y0 + (int)(c >> 8 & 255u) - (1 << P::LY)) < my &&
+         (uint32_t)(z0 + (int)(c >> 16) - (1 << P::LZ)) < mz;
+}
+// (A policy's cells() replaces the words that are not kNoMark.)
+// the word of the end of a path: the node that mark_ends gave the cell (ends
+// that are not in the list have none: bad data)
+__device__ __forceinline__ uint32_t end_word(const uint32_t* path, int64_t cell, const int64_t* list,
+                                             int64_t n, uint32_t node0) {
+  const uint32_t w = path[cell];
+  const int64_t i = (int64_t)(w & ~kEnd) - node0;
+  return (w & kEnd) && i >= 0 && i < n && __ldg(list + i) == cell ? w : kNoMark;
+}
+
+// D0: descending paths from vertex to vertex, to a minimum
 template <class F>
-struct DescWalk {
+struct DescPaths {
+  static constexpr int K = 1, LX = 4, LY = 4, LZ = 4;
   F fields;
-  const int64_t* crit1;
   const uint8_t* desc;
-  uint32_t* claim;
-  struct State {
-    Grid g;
-    int64_t v, it;
-  };
-  // start walk j of saddle s; false if it has already ended (never, here)
-  __device__ __forceinline__ bool start(int64_t s, int j, State& st, uint32_t& r) const {
-    const int64_t id = crit1[s];
-    const int64_t a = id / 7;
-    const int k = (int)(id - a * 7);
-    int64_t off;
-    fields.get(a, st.g, off);
-    st.v = j ? a + corner_delta(st.g, edge_corner(k)) : a;
-    st.it = 0;
-    (void)r;
-    return true;
-  }
-  // one step; false when the walk has ended with result r.  The gradient
-  // load and the claim of the current vertex are in flight together; the
-  // minima carry end marks, so a walk learns its end from the failed claim
-  __device__ __forceinline__ bool step(State& st, uint32_t w, uint32_t& r,
-                                       int32_t* dstatus) const {
-    const uint8_t d = __ldg(desc + st.v);
-    const uint32_t old = atomicCAS(claim + st.v, kUnclaimed, w);
-    if (old != kUnclaimed) {
-      r = claim_result(old);
-      return false;
+  const int64_t* ends;  // the path ends' cells, their number (n_dev or n)
+  const int64_t* n_dev;
+  int64_t n;
+  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
+                                        int y0, int z0, bool border, uint32_t (&w)[K]) const {
+    const int d = __ldg(desc + v);
+    if (d >= 14) {
+      if (d == 15) w[0] = end_word(path, v, ends, n_dev ? *n_dev : n, 0);
+      return;
     }
-    if (d >= 14) {  // a minimum without its end mark: inconsistent input
-      set_status(dstatus, DMS_ERR_ARG);
-      r = 0;
-      return false;
-    }
-    st.v += slot_delta_g(st.g, d);
-    if (++st.it > st.g.n) {
-      set_status(dstatus, DMS_ERR_TIMEOUT);
-      r = 0;
-      return false;
-    }
-    return true;
+    const int c = (0x7653421 >> (4 * (d < 7 ? d : d - 7))) & 15, s = d < 7 ? 1 : -1;
+    const uint32_t to = packed_coords<DescPaths>(lv) +
+                        s * packed_step(c & 1, (c >> 1) & 1, (c >> 2) & 1);
+    const bool out = border && !inside<DescPaths>(to, x0, y0, z0, (uint32_t)g.nx, (uint32_t)g.ny, (uint32_t)g.nz);
+    if (!out) w[0] = brick_word<DescPaths>(to, 0);  // (outside: bad data)
   }
 };
 
-// D2: ascending dual paths from the two cofacets of a critical triangle to a
-// critical tetrahedron (node j + 1) or out of the grid (node 0, OUTSIDE)
+// the steps of the dual paths from tet type k with code c, at 4 k + c - 1, and
+// the type they lead to (codes 2 and 3 stay at the anchor)
+struct DualSteps {
+  uint32_t step[24];
+  uint8_t type[24];
+};
+constexpr DualSteps make_dual_steps() {
+  DualSteps t{};
+  for (int e = 0; e < 24; ++e) {
+    const uint64_t w = dual_step_detail::entry(e);
+    const int c = (int)(w >> 3) & 7, sg = (int)(w >> 6) == 1 ? 1 : ((int)(w >> 6) == 2 ? -1 : 0);
+    t.step[e] = (uint32_t)(sg * ((c & 1) + ((c >> 1) & 1) * 256 + ((c >> 2) & 1) * 65536));
+    t.type[e] = (uint8_t)(w & 7);
+  }
+  return t;
+}
+
+// D2: ascending dual paths from tet to tet, to a critical one or out of the
+// grid (node 0, OUTSIDE)
 template <class F>
-struct DualWalk {
+struct DualPaths {
+  static constexpr int K = 6, LX = 4, LY = 3, LZ = 3;
   F fields;
-  const int64_t* crit2;
   const uint64_t* rec;
-  uint32_t* claim;
-  // the walk's tet (anchor b, type k), the anchor's coordinates and the
-  // grid's strides and bounds in 32-bit form where they fit
-  struct State {
-    int64_t b, sy, sz;
-    int bx, by, bz, k;
-    uint32_t mx, my, mz;  // dims - 1: a tet anchor lies below them in every axis
-    uint32_t it, lim;
-  };
-  __device__ __forceinline__ bool start(int64_t s, int j, State& st, uint32_t& r) const {
-    const int64_t id = crit2[s];
-    const int64_t a = id / 12;
-    const int k = (int)(id - a * 12);
-    Grid g;
-    int64_t off;
-    fields.get(a, g, off);
-    int64_t ax, ay, az;
-    fields.coords(g, a - off, ax, ay, az);
-    int64_t cof[2];
-    tri_cofacets(g, a, k, ax, ay, az, cof);
-    const int64_t t = j ? cof[1] : cof[0];
-    if (t < 0) {
-      r = 0;  // no cofacet on that side: the walk starts OUTSIDE
-      return false;
+  const int64_t* ends;
+  const int64_t* n_dev;
+  int64_t n;
+  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
+                                        int y0, int z0, bool border, uint32_t (&w)[K]) const {
+    constexpr DualSteps st = make_dual_steps();
+    const uint32_t hi = (uint32_t)(__ldg(rec + v) >> 32), at = packed_coords<DualPaths>(lv);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const uint32_t code = (hi >> (1 + 3 * k)) & 7u;
+      if (code == 7u) {
+        w[k] = end_word(path, v * 6 + k, ends, n_dev ? *n_dev : n, 1);
+      } else if (code >= 1u && code <= 4u) {  // (else no tet there, or bad data)
+        const uint32_t to = at + (code == 1u ? st.step[4 * k] : (code == 4u ? st.step[4 * k + 3] : 0u));
+        const int t = code == 1u ? st.type[4 * k] : (code == 2u ? st.type[4 * k + 1]
+                                                  : (code == 3u ? st.type[4 * k + 2] : st.type[4 * k + 3]));
+        // (tet anchors lie below the last vertex in every axis)
+        const bool out = border && !inside<DualPaths>(to, x0, y0, z0, (uint32_t)(g.nx - 1),
+                                                      (uint32_t)(g.ny - 1), (uint32_t)(g.nz - 1));
+        w[k] = out ? kEnd : brick_word<DualPaths>(to, t);  // out: OUTSIDE
+      }
     }
-    st.b = t / 6;
-    st.k = (int)(t - st.b * 6);
-    int64_t bx, by, bz;
-    fields.coords(g, st.b - off, bx, by, bz);
-    st.bx = (int)bx;
-    st.by = (int)by;
-    st.bz = (int)bz;
-    st.sy = g.nx;
-    st.sz = g.sxy;
-    st.mx = (uint32_t)(g.nx - 1);
-    st.my = (uint32_t)(g.ny - 1);
-    st.mz = (uint32_t)(g.nz - 1);
-    st.it = 0;
-    st.lim = (uint32_t)min(6 * g.n, (int64_t)0xFFFFFFFF);
-    return true;
-  }
-  // record load and claim in flight together, as for the descending walks;
-  // the critical tets carry end marks
-  __device__ __forceinline__ bool step(State& st, uint32_t w, uint32_t& r,
-                                       int32_t* dstatus) const {
-    const uint64_t rw = __ldg(rec + st.b);
-    const uint32_t old = atomicCAS(claim + st.b * 6 + st.k, kUnclaimed, w);
-    if (old != kUnclaimed) {
-      r = claim_result(old);
-      return false;
-    }
-    const uint32_t code = (uint32_t)(rw >> (33 + 3 * st.k)) & 7u;
-    if (code < 1u || code > 4u) {  // a critical tet without its end mark, or bad data
-      set_status(dstatus, DMS_ERR_ARG);
-      r = 0;
-      return false;
-    }
-    // the next tet, without branching on the code (lanes take different
-    // codes): a zero step leaves the anchor where it is
-    const uint32_t t = dual_step(st.k, code);
-    const int stp = (int)((t >> 3) & 7u);
-    const int sg = (t >> 6) == 1u ? 1 : ((t >> 6) == 2u ? -1 : 0);
-    st.bx += sg * (stp & 1);
-    st.by += sg * ((stp >> 1) & 1);
-    st.bz += sg * ((stp >> 2) & 1);
-    // the anchor of a tet needs +1 inside in every axis (negative -> huge)
-    if ((uint32_t)st.bx >= st.mx || (uint32_t)st.by >= st.my || (uint32_t)st.bz >= st.mz) {
-      r = 0;  // left the grid: OUTSIDE
-      return false;
-    }
-    const int64_t d = (int64_t)(stp & 1) + (((stp >> 1) & 1) ? st.sy : 0) + (((stp >> 2) & 1) ? st.sz : 0);
-    st.b += sg * d;
-    st.k = (int)(t & 7u);
-    if (++st.it > st.lim) {
-      set_status(dstatus, DMS_ERR_TIMEOUT);
-      r = 0;
-      return false;
-    }
-    return true;
   }
 };
 
-// Both walks of every saddle, taken from a queue by the lanes of a
-// persistent grid: a lane whose walk has ended takes the next walk id, so
-// that one long walk no longer holds the other 31 lanes of its warp idle
-// (with a saddle per thread, 5-6 lanes of 32 were active on average).  The
-// walks are chains of dependent loads, and the number in flight is what
-// hides their latency.  A warp takes ids from the shared cursor in blocks of
-// kWalkBlock (one atomic per block, not per walk) and deals them out to its
-// lanes in order.  Walk w is walk w & 1 of saddle w >> 1; the walks of one
-// saddle may run at the same time, which the claims allow (see above).
-constexpr uint32_t kWalkBlock = 256;
-
-__device__ __forceinline__ void store_walk(Tri T, uint32_t w, uint32_t r) {
-  if (w & 1) T.s[w >> 1].rb = r;
-  else T.s[w >> 1].ra = r;
-}
-
-template <class W>
-__global__ void __launch_bounds__(256) walk_queue(const W wk, const int64_t* n_dev, int64_t n_host,
-                                                  unsigned int* cursor, Tri T, int32_t* dstatus) {
-  const int64_t ns = n_dev ? *n_dev : n_host;
-  const uint32_t nwalks = (uint32_t)(2 * ns);  // < 2^31: walk ids sit below kLinkBit
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  uint32_t qnext = 0, qend = 0;  // this warp's block of walk ids (warp-uniform)
-  uint32_t cur = kNone;          // the lane's walk, kNone between walks
-  bool done = false;             // no walk left for this lane
-  typename W::State st;
-  for (;;) {
-    const bool need = !done && cur == kNone;
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, need);
-    if (m) {
-      const uint32_t k = (uint32_t)__popc(m), i = (uint32_t)__popc(m & lt);
-      uint32_t nbase = 0;
-      if (qnext + k > qend) {  // the block runs out: take the next one
-        if (lane == 0) nbase = atomicAdd(cursor, kWalkBlock);
-        nbase = __shfl_sync(0xFFFFFFFFu, nbase, 0);
+// One CTA per brick: the words of all its cells, by pointer doubling.  A word
+// is always a cell further along the path, so no barrier is needed between
+// passes: every thread goes on until its own words are final.  (A path that
+// loops, of bad data, is left as kLoop after as many passes as the brick has
+// cells.)
+constexpr int kBrickThreads = 256;
+template <class P>
+__global__ void __launch_bounds__(kBrickThreads) resolve_paths(const P p, uint32_t* path) {
+  constexpr int VERTS = 1 << (P::LX + P::LY + P::LZ), CELLS = VERTS * P::K;
+  static_assert(CELLS <= 8192, "a cell of a brick has 13 bits");
+  __shared__ uint32_t s[CELLS];
+  volatile uint32_t* const vs = s;
+  Grid g;
+  int64_t off;
+  int bx, by, bz;
+  p.fields.brick(blockIdx.x, P::LX, P::LY, P::LZ, g, off, bx, by, bz);
+  const int x0 = bx << P::LX, y0 = by << P::LY, z0 = bz << P::LZ;
+  const int wx = min((int64_t)1 << P::LX, g.nx - x0), wy = min((int64_t)1 << P::LY, g.ny - y0);
+  const int wz = min((int64_t)1 << P::LZ, g.nz - z0);
+  // a step from this brick may leave the grid (or reach its last vertices,
+  // which anchor no tets)
+  const bool border = bx == 0 || by == 0 || bz == 0 || x0 + (1 << P::LX) >= g.nx - 1 ||
+                      y0 + (1 << P::LY) >= g.ny - 1 || z0 + (1 << P::LZ) >= g.nz - 1;
+  const int64_t first = off + x0 + g.nx * y0 + g.sxy * z0;
+  // a thread's words stay in registers, too
+  constexpr int VPT = VERTS / kBrickThreads;
+  uint32_t w[VPT][P::K];
+#pragma unroll
+  for (int j = 0; j < VPT; ++j) {
+    const int lv = j * kBrickThreads + threadIdx.x;
+    const int lx = lv & ((1 << P::LX) - 1), ly = (lv >> P::LX) & ((1 << P::LY) - 1), lz = lv >> (P::LX + P::LY);
+#pragma unroll
+    for (int k = 0; k < P::K; ++k) w[j][k] = kNoMark;
+    if (lx < wx && ly < wy && lz < wz)
+      p.cells(g, path, first + lx + g.nx * ly + g.sxy * lz, lv, x0, y0, z0, border, w[j]);
+#pragma unroll
+    for (int k = 0; k < P::K; ++k) vs[lv * P::K + k] = w[j][k];
+  }
+  __syncthreads();
+  bool again = true;
+  for (int pass = 0; again && pass < CELLS; ++pass) {
+    again = false;
+#pragma unroll
+    for (int j = 0; j < VPT; ++j)
+#pragma unroll
+      for (int k = 0; k < P::K; ++k) {
+        if (w[j][k] & (kEnd | kFinal)) continue;
+        w[j][k] = vs[w[j][k]];
+        vs[(j * kBrickThreads + threadIdx.x) * P::K + k] = w[j][k];
+        again = true;
       }
-      if (need) {
-        const uint32_t w = qnext + i < qend ? qnext + i : nbase + (qnext + i - qend);
-        if (w < nwalks) {
-          uint32_t r = 0;
-          if (wk.start((int64_t)(w >> 1), (int)(w & 1), st, r)) cur = w;
-          else store_walk(T, w, r);
-        } else {
-          done = true;
-        }
-      }
-      if (qnext + k > qend) {
-        qnext = nbase + (qnext + k - qend);
-        qend = nbase + kWalkBlock;
-      } else {
-        qnext += k;
-      }
+  }
+  if (again) {  // bad data: a path that loops
+#pragma unroll
+    for (int j = 0; j < VPT; ++j)
+#pragma unroll
+      for (int k = 0; k < P::K; ++k)
+        if (!(w[j][k] & (kEnd | kFinal))) vs[(j * kBrickThreads + threadIdx.x) * P::K + k] = kLoop;
+  }
+  __syncthreads();
+  // rows of vertices, whose cells are consecutive here and in memory, to warps
+  constexpr int ROW = P::K << P::LX, ROWS = VERTS >> P::LX;
+  for (int row = threadIdx.x >> 5; row < ROWS; row += kBrickThreads / 32) {
+    const int ly = row & ((1 << P::LY) - 1), lz = row >> P::LY;
+    if (ly >= wy || lz >= wz) continue;
+    uint32_t* out = path + (first + g.nx * ly + g.sxy * lz) * P::K;
+#pragma unroll
+    for (int c = threadIdx.x & 31; c < ROW; c += 32) {
+      const uint32_t w = s[row * ROW + c];
+      if (c < wx * P::K) out[c] = w & kEnd ? w : w & ~kFinal;
     }
-    if (cur != kNone) {
-      uint32_t r = 0;
-      if (!wk.step(st, cur, r, dstatus)) {
-        // joined another walk: take its result if it is already known (its
-        // end node, or a link one hop further), so that link_walks has
-        // fewer links to follow; a pending one (kNone) keeps the link
-        if (r & kLinkBit) {
-          const uint32_t w2 = r & ~kLinkBit;
-          const uint32_t r2 = (w2 & 1) ? T.s[w2 >> 1].rb : T.s[w2 >> 1].ra;
-          if (r2 != kNone) r = r2;
-        }
-        store_walk(T, cur, r);
-        cur = kNone;
-      }
-    }
-    if (__all_sync(0xFFFFFFFFu, done)) break;
   }
 }
 
-// the walks of n saddles (count on the device when n_dev is given); cursor
-// is a zeroed device word
-template <class W>
-int launch_walks(const W& wk, const int64_t* n_dev, int64_t n_host, unsigned int* cursor, Tri T,
-                 int32_t* dstatus, cudaStream_t s) {
-  static int blocks = 0;
-  if (blocks == 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_queue<W>, 256, 0) !=
-            cudaSuccess)
-      return DMS_ERR_CUDA;
-    blocks = std::max(1, sms * std::max(1, per_sm));
-  }
-  unsigned g = (unsigned)blocks;
-  if (!n_dev) g = (unsigned)std::min<int64_t>(g, (2 * n_host + 255) / 256 + 1);
-  walk_queue<<<g, 256, 0, s>>>(wk, n_dev, n_host, cursor, T, dstatus); count_launch();
-  return DMS_OK;
+template <class P>
+int64_t brick_count(int64_t nx, int64_t ny, int64_t nz) {
+  return ((nx + (1 << P::LX) - 1) >> P::LX) * ((ny + (1 << P::LY) - 1) >> P::LY) *
+         ((nz + (1 << P::LZ) - 1) >> P::LZ);
 }
 
-// Second pass (D0 and D2): resolve both walks of each saddle to their end
-// nodes; a saddle whose walks end at different nodes is live in the pairing.
-// (saddles marked in Sad::pad are left out of the pairing: on 2D grids the
-// D1 pass skips the edges D0 already paired).  With tag set it also does the
-// first round's search of the pairing rounds (round_find, round 1: every
-// node is still its own root): it records both ends as the roots and tags
-// them with the saddle, so that the rounds start at their merge step.  (A
-// resolver reading ra / rb of a saddle while it is overwritten gets the
-// walk's end node either way.)
-__global__ void __launch_bounds__(256) link_walks(int64_t nt, Tri T, uint32_t* live,
-                                                  unsigned int* live_n, int32_t* dstatus,
-                                                  bool skip_marked = false, bool tag = false,
-                                                  Nodes nd = Nodes{}) {
+// a walk: the word of its cell and the brick of that cell
+struct Walk {
+  uint32_t w;
+  int bx, by, bz;
+};
+template <class P>
+__device__ __forceinline__ Walk walk_from(const uint32_t* path, const Grid& g, int64_t v, int x, int y, int z,
+                                          int k) {
+  return Walk{__ldg(path + v * P::K + k), x >> P::LX, y >> P::LY, z >> P::LZ};
+}
+template <class P>
+__device__ __forceinline__ void walk_hop(const uint32_t* path, const Grid& g, int64_t off, Walk& a) {
+  const uint32_t local = a.w & 8191u, lv = local / P::K;
+  a.bx += (int)(a.w >> 13 & 3u) - 1;
+  a.by += (int)(a.w >> 15 & 3u) - 1;
+  a.bz += (int)(a.w >> 17 & 3u) - 1;
+  const int x = (a.bx << P::LX) + (int)(lv & ((1 << P::LX) - 1));
+  const int y = (a.by << P::LY) + (int)((lv >> P::LX) & ((1 << P::LY) - 1));
+  const int z = (a.bz << P::LZ) + (int)(lv >> (P::LX + P::LY));
+  a.w = __ldg(path + (off + x + g.nx * y + g.sxy * z) * P::K + (local - lv * P::K));
+}
+__device__ __forceinline__ uint32_t walk_end(const Walk& a, int32_t* dstatus) {
+  if (a.w < kLoop) return a.w & ~kEnd;
+  set_status(dstatus, a.w == kLoop ? DMS_ERR_TIMEOUT : DMS_ERR_ARG);  // bad data
+  return 0;
+}
+// both walks of a saddle to their ends, their loads in flight together (a
+// path through more bricks than there are cells loops: bad data)
+template <class P>
+__device__ __forceinline__ void walk_both(const uint32_t* path, const Grid& g, int64_t off, Walk& a, Walk& b) {
+  int64_t left = g.n * P::K;
+  while (!(a.w & kEnd) || !(b.w & kEnd)) {
+    if (!(a.w & kEnd)) walk_hop<P>(path, g, off, a);
+    if (!(b.w & kEnd)) walk_hop<P>(path, g, off, b);
+    if (--left < 0) {
+      a.w = a.w & kEnd ? a.w : kLoop;
+      b.w = b.w & kEnd ? b.w : kLoop;
+    }
+  }
+}
+
+// the saddle's record with its weight and ends, live where they differ.  With
+// tag set it also does the first round's search of the pairing rounds (every
+// node is still its own root): both ends are the roots and are tagged with the
+// saddle, so that the rounds start at their merge step.
+__device__ __forceinline__ bool store_saddle(Tri T, int64_t i, uint64_t w, uint32_t n0, uint32_t n1,
+                                             bool tag, const Nodes& nd) {
+  Sad sd;
+  sd.w = w;
+  sd.na = sd.ra = n0;
+  sd.nb = sd.rb = n1;
+  sd.res = kNone;
+  sd.pad = 0;
+  T.s[i] = sd;
+  if (n0 == n1) return false;
+  if (tag) {
+    const unsigned long long tv = (1ull << 44) | (kMask44 - w);
+    if (n0 != nd.immortal) atomicMax(nd.best + n0, tv);
+    if (n1 != nd.immortal) atomicMax(nd.best + n1, tv);
+  }
+  return true;
+}
+
+// ranks of two neighbours u1, u2 (orders o1, o2) of vertex t = (x, y, z) of a
+// field among the neighbours of t below
+__device__ __forceinline__ void star_ranks(const Grid& g, const uint32_t* __restrict__ order, int64_t t,
+                                           int x, int y, int z, uint32_t o1, uint32_t o2,
+                                           uint32_t& r1, uint32_t& r2) {
+  const int mx = (int)g.nx, my = (int)g.ny, mz = (int)g.nz;
+  r1 = r2 = 0;
+#pragma unroll
+  for (int s = 0; s < 14; ++s) {
+    const int c = (0x7653421 >> (4 * (s < 7 ? s : s - 7))) & 15;
+    const int sg = s < 7 ? 1 : -1;
+    const int nx = x + sg * (c & 1), ny = y + sg * ((c >> 1) & 1), nz = z + sg * ((c >> 2) & 1);
+    if ((uint32_t)nx >= (uint32_t)mx || (uint32_t)ny >= (uint32_t)my || (uint32_t)nz >= (uint32_t)mz) continue;
+    const uint32_t on = __ldg(order + t + slot_delta_g(g, s));
+    r1 += on < o1 ? 1u : 0u;
+    r2 += on < o2 ? 1u : 0u;
+  }
+}
+
+// D0: each critical edge's weight (its lexicographic key), its two descending
+// paths.  (Bound by random reads of orders and path words: 32 registers for 64
+// warps an SM; the D0/D2 stage of 1024^3 takes 80.3 ms with 54, 76.6 with 32.)
+template <class F>
+__global__ void __launch_bounds__(256, 8) link_d0(const F fields, const uint32_t* __restrict__ order,
+                                               const int64_t* __restrict__ crit1,
+                                               const int64_t* n_dev, int64_t n_host,
+                                               const uint32_t* __restrict__ path, Tri T,
+                                               uint32_t* live, unsigned int* live_n,
+                                               int32_t* dstatus, bool tag, Nodes nd) {
   __shared__ CtaAppend sh;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  bool keep = false;
-  if (i < nt && !(skip_marked && T.s[i].pad)) {
-    const uint32_t n0 = resolve_walk(T.s, T.s[i].ra, 2 * nt, dstatus);
-    const uint32_t n1 = resolve_walk(T.s, T.s[i].rb, 2 * nt, dstatus);
-    if (n0 != n1) {
-      T.s[i].na = n0;
-      T.s[i].nb = n1;
-      keep = true;
-      if (tag) {
-        T.s[i].ra = n0;
-        T.s[i].rb = n1;
-        const unsigned long long tv = (1ull << 44) | (kMask44 - T.s[i].w);
-        if (n0 != nd.immortal) atomicMax(nd.best + n0, tv);
-        if (n1 != nd.immortal) atomicMax(nd.best + n1, tv);
-      }
+  const int64_t ne = n_dev ? *n_dev : n_host;
+  // CTA-uniform passes: every thread reaches the appends
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < ne;
+       base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = base + threadIdx.x;
+    bool keep = false;
+    if (i < ne) {
+      const int64_t id = crit1[i], a = id / 7;
+      const int c = edge_corner((int)(id - a * 7));
+      Grid g;
+      int64_t off;
+      fields.get(a, g, off);
+      int x, y, z;
+      coords(g, a - off, x, y, z);
+      const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
+      const int64_t b = a + corner_delta(g, c);
+      Walk wa = walk_from<DescPaths<F>>(path, g, a, x, y, z, 0);
+      Walk wb = walk_from<DescPaths<F>>(path, g, b, x + cx, y + cy, z + cz, 0);
+      const uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
+      const bool up = ob > oa;
+      uint32_t r, r2;
+      star_ranks(g, order, up ? b : a, up ? x + cx : x, up ? y + cy : y, up ? z + cz : z, min(oa, ob),
+                 min(oa, ob), r, r2);
+      walk_both<DescPaths<F>>(path, g, off, wa, wb);
+      keep = store_saddle(T, i, ((uint64_t)(oa > ob ? oa : ob) << 4) | r, walk_end(wa, dstatus),
+                          walk_end(wb, dstatus), tag, nd);
     }
+    cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
   }
-  cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+}
+
+// D2: each critical triangle's weight (decreasing triangle key), the two dual
+// paths from its cofacets
+template <class F>
+__global__ void __launch_bounds__(256, 8) link_d2(const F fields, const uint32_t* __restrict__ order,
+                                               const int64_t* __restrict__ crit2,
+                                               const int64_t* n_dev, int64_t n_host,
+                                               const uint32_t* __restrict__ path, Tri T,
+                                               uint32_t* live, unsigned int* live_n,
+                                               int32_t* dstatus, bool tag, Nodes nd) {
+  __shared__ CtaAppend sh;
+  const int64_t nt = n_dev ? *n_dev : n_host;
+  // CTA-uniform passes: every thread reaches the appends
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < nt;
+       base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = base + threadIdx.x;
+    bool keep = false;
+    if (i < nt) {
+      const int64_t id = crit2[i], a = id / 12;
+      const int k = (int)(id - a * 12);
+      Grid g;
+      int64_t off, cof[2];
+      fields.get(a, g, off);
+      int x, y, z;
+      coords(g, a - off, x, y, z);
+      tri_cofacets(g, a, k, x, y, z, cof);
+      Walk wk[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (cof[j] < 0) {
+          wk[j] = Walk{kEnd, 0, 0, 0};  // no cofacet on that side: OUTSIDE
+        } else {
+          const int64_t v = cof[j] / 6;
+          int vx, vy, vz;
+          coords(g, v - off, vx, vy, vz);
+          wk[j] = walk_from<DualPaths<F>>(path, g, v, vx, vy, vz, (int)(cof[j] - v * 6));
+        }
+      }
+      // the key: the order of the highest vertex, the ranks of the others
+      // among its neighbours
+      const int c[3] = {0, tri_p(k), tri_q(k)};
+      uint32_t o[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) o[j] = __ldg(order + a + corner_delta(g, c[j]));
+      int it = 0;
+      if (o[1] > o[it]) it = 1;
+      if (o[2] > o[it]) it = 2;
+      uint32_t om = 0, ol = 0xFFFFFFFFu;
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (j != it) {
+          om = max(om, o[j]);
+          ol = min(ol, o[j]);
+        }
+      const int ct = it == 0 ? 0 : (it == 1 ? c[1] : c[2]);
+      uint32_t rm, rl;
+      star_ranks(g, order, a + corner_delta(g, ct), x + (ct & 1), y + ((ct >> 1) & 1),
+                 z + ((ct >> 2) & 1), om, ol, rm, rl);
+      const uint64_t key = ((uint64_t)max(o[0], max(o[1], o[2])) << 8) | (rm << 4) | rl;
+      walk_both<DualPaths<F>>(path, g, off, wk[0], wk[1]);
+      keep = store_saddle(T, i, kMask44 - key, walk_end(wk[0], dstatus), walk_end(wk[1], dstatus), tag, nd);
+    }
+    cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+  }
 }
 
 __global__ void init_nodes_d0(const uint32_t* __restrict__ order, const int64_t* __restrict__ crit0,
@@ -871,7 +926,6 @@ enum : int {
   kCtrForest = 2,    // saddles of the spanning forest
   kCtrChanged = 3,   // (self-correcting pairing)
   kCtrBig = 4,       // saddles left to the device-wide sorted finish (batch)
-  kCtrWalk = 6,      // walk cursor
   kCtrRound = 8,     // three live counts in turn
   kCtrLeft = 11,     // saddles left live by the exact rounds
   kCtrBarrier = 12,
@@ -889,7 +943,7 @@ struct Rounds {
   // rounds); then, unless forest_only, the exact rounds on them follow
   uint32_t* forest;
   bool forest_only;
-  bool first_found;       // the first round's search is done (link_walks)
+  bool first_found;       // the first round's search is done (link_d0, link_d2)
   unsigned int* ctr;
   const int64_t* n_dev;   // node count: *n_dev + nnode, or nnode alone
   int64_t nnode;
@@ -1293,15 +1347,14 @@ struct DiagWs {
   // nd.parent and nd.best)
   uint32_t* sc_parent;
   unsigned long long* sc_w;
-  uint32_t* claim;  // one word per tet id: the dual walk that passed it
-  int64_t nclaim;
+  uint32_t* path;  // one word per cell (vertex / tet id): where its path goes on or ends
   radix64::Buffers rb;
   size_t bytes;
 };
 
 // nc: counts of the node and saddle lists as for 3D (minima, edges, triangles,
-// tets); nclaim: claim words, one per vertex / tet id the walks may visit
-DiagWs carve_diag(void* base, const int64_t* nc, int64_t nclaim) {
+// tets); npath: path words, one per vertex / tet id the walks may visit
+DiagWs carve_diag(void* base, const int64_t* nc, int64_t npath) {
   WsCarver c(base);
   DiagWs w;
   const int64_t nsad = std::max<int64_t>(std::max<int64_t>(nc[1], nc[2]), 1);
@@ -1319,8 +1372,7 @@ DiagWs carve_diag(void* base, const int64_t* nc, int64_t nclaim) {
   w.nd.immortal = kNone;
   w.sc_parent = c.take<uint32_t>(nnode);
   w.sc_w = c.take<unsigned long long>(nnode);
-  w.nclaim = nclaim;
-  w.claim = c.take<uint32_t>(w.nclaim);
+  w.path = c.take<uint32_t>(npath);
   w.rb = radix64::carve(c, std::max<int64_t>(nsad, 4096));
   w.bytes = c.used;
   return w;
@@ -1594,17 +1646,15 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
     init_nodes_d0<<<nb(nc[0]), TB, 0, s>>>(order, crit0, nc[0], w.nd); count_launch();
     write_essential<<<nb(nc[0]), TB, 0, s>>>(f, order, crit0, nc[0], ess); count_launch();
   }
+  w.nd.immortal = kNone;  // every minimum but the global one can die
   if (nc[1] > 0) {
-    DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, g.n * sizeof(uint32_t), s));
-    mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.claim); count_launch();
-    d0_weights<<<nb(nc[1]), TB, 0, s>>>(D, order, crit1, nc[1], w.T0); count_launch();
-    const DescWalk<OneField> wk{OneField{g}, crit1, desc, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, nc[1], w.ctr + kCtrWalk, w.T0, dstatus, s));
-    w.nd.immortal = kNone;  // every minimum but the global one can die
-    link_walks<<<nb(nc[1]), TB, 0, s>>>(nc[1], w.T0, w.live0, w.ctr + kCtrLive, dstatus, false,
-                                        pairing == 0, w.nd); count_launch();
+    const DescPaths<OneField> paths{OneField{g}, desc, crit0, nullptr, nc[0]};
+    mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.path); count_launch();
+    resolve_paths<<<(unsigned)brick_count<DescPaths<OneField>>(g.nx, g.ny, g.nz), kBrickThreads, 0, s>>>(
+        paths, w.path); count_launch();
+    link_d0<<<nb(nc[1]), TB, 0, s>>>(OneField{g}, order, crit1, nullptr, nc[1], w.path, w.T0, w.live0,
+                                     w.ctr + kCtrLive, dstatus, pairing == 0, w.nd); count_launch();
   }
-  w.nd.immortal = kNone;
   int st = pairing == 1 ? run_selfcorrecting(w, w.T0, std::max<int64_t>(nc[0], 1), s, dstatus)
                         : run_pairing(w, w.T0, nc[1], std::max<int64_t>(nc[0], 1), s, dstatus, true);
   if (st) return st;
@@ -1614,19 +1664,17 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
   // ---- D2
   DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   init_nodes_d2<<<nb(nc[3] + 1), TB, 0, s>>>(D, order, crit3, nc[3], w.nd); count_launch();
+  w.nd.immortal = 0;  // OUTSIDE
   if (nc[2] > 0) {
-    DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, w.nclaim * sizeof(uint32_t), s));
+    const DualPaths<OneField> paths{OneField{g}, rec, crit3, nullptr, nc[3]};
     if (nc[3] > 0) {
-      mark_ends<<<nb(nc[3]), TB, 0, s>>>(crit3, nullptr, nc[3], 1, w.claim); count_launch();
+      mark_ends<<<nb(nc[3]), TB, 0, s>>>(crit3, nullptr, nc[3], 1, w.path); count_launch();
     }
-    d2_weights<<<nb(nc[2]), TB, 0, s>>>(D, order, crit2, nc[2], w.T2); count_launch();
-    const DualWalk<OneField> wk{OneField{g}, crit2, rec, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, nc[2], w.ctr + kCtrWalk, w.T2, dstatus, s));
-    w.nd.immortal = 0;  // OUTSIDE
-    link_walks<<<nb(nc[2]), TB, 0, s>>>(nc[2], w.T2, w.live0, w.ctr + kCtrLive, dstatus, false,
-                                        pairing == 0, w.nd); count_launch();
+    resolve_paths<<<(unsigned)brick_count<DualPaths<OneField>>(g.nx, g.ny, g.nz), kBrickThreads, 0, s>>>(
+        paths, w.path); count_launch();
+    link_d2<<<nb(nc[2]), TB, 0, s>>>(OneField{g}, order, crit2, nullptr, nc[2], w.path, w.T2, w.live0,
+                                     w.ctr + kCtrLive, dstatus, pairing == 0, w.nd); count_launch();
   }
-  w.nd.immortal = 0;
   st = pairing == 1 ? run_selfcorrecting(w, w.T2, nc[3] + 1, s, dstatus)
                     : run_pairing(w, w.T2, nc[2], nc[3] + 1, s, dstatus, true);
   if (st) return st;
@@ -1731,27 +1779,6 @@ __global__ void b_essential(const FieldTab ft, const float* __restrict__ f,
   }
 }
 
-__global__ void b_d0_weights(const FieldTab ft, const uint32_t* __restrict__ order,
-                             const int64_t* __restrict__ crit1, const int64_t* __restrict__ cnt,
-                             Tri T) {
-  const int64_t ne = cnt[1];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ne;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t id = crit1[i];
-    const int64_t a = id / 7;
-    const int k = (int)(id - a * 7);
-    const dms_field_desc fd = ft.fd[field_of_vertex(ft, a)];
-    const Grid g = grid_of(fd);
-    const int64_t b = a + corner_delta(g, edge_corner(k));
-    const uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
-    const int64_t top = oa > ob ? a : b;
-    const uint32_t r = local_rank_f(g, fd.offset, order, top, oa > ob ? ob : oa);
-    T.s[i].w = ((uint64_t)(oa > ob ? oa : ob) << 4) | r;
-    T.s[i].res = kNone;
-    T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
-  }
-}
-
 __global__ void b_init_nodes_d2(const FieldTab ft, const uint32_t* __restrict__ order,
                                 const int64_t* __restrict__ crit3, const int64_t* __restrict__ cnt,
                                 Nodes nd) {
@@ -1789,66 +1816,17 @@ __global__ void b_init_nodes_d2(const FieldTab ft, const uint32_t* __restrict__ 
   }
 }
 
-__global__ void b_d2_weights(const FieldTab ft, const uint32_t* __restrict__ order,
-                             const int64_t* __restrict__ crit2, const int64_t* __restrict__ cnt,
-                             Tri T) {
-  const int64_t nt = cnt[2];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nt;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t id = crit2[i];
-    const int64_t a = id / 12;
-    const int k = (int)(id - a * 12);
-    const dms_field_desc fd = ft.fd[field_of_vertex(ft, a)];
-    const Grid g = grid_of(fd);
-    const int p = tri_p(k), q = tri_q(k);
-    int64_t v[3] = {a, a + corner_delta(g, p), a + corner_delta(g, q)};
-    uint32_t o[3] = {__ldg(order + v[0]), __ldg(order + v[1]), __ldg(order + v[2])};
-    int it = 0;
-    if (o[1] > o[it]) it = 1;
-    if (o[2] > o[it]) it = 2;
-    uint32_t om = 0, ol = 0xFFFFFFFFu;
-    for (int j = 0; j < 3; ++j)
-      if (j != it) {
-        om = max(om, o[j]);
-        ol = min(ol, o[j]);
-      }
-    const uint32_t rm = local_rank_f(g, fd.offset, order, v[it], om);
-    const uint32_t rl = local_rank_f(g, fd.offset, order, v[it], ol);
-    const uint64_t key = ((uint64_t)o[it] << 8) | (rm << 4) | rl;
-    T.s[i].w = kMask44 - key;
-    T.s[i].res = kNone;
-    T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
+// the fields' first bricks (one small CTA): fields in turn, a few hundred
+__global__ void brick_table(const FieldTab ft, int lx, int ly, int lz, int64_t* brick0) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  int64_t acc = 0;
+  for (int f = 0; f < ft.n; ++f) {
+    brick0[f] = acc;
+    const dms_field_desc d = ft.fd[f];
+    acc += (int64_t)((d.nx + (1 << lx) - 1) >> lx) * ((d.ny + (1 << ly) - 1) >> ly) *
+           ((d.nz + (1 << lz) - 1) >> lz);
   }
-}
-
-// As link_walks with tag set: also the forest's first round search (both
-// ends recorded as roots and tagged), so the rounds start at their hook.
-__global__ void __launch_bounds__(256) b_link_walks(const int64_t* __restrict__ n_dev, Tri T,
-                                                    uint32_t* live, unsigned int* live_n,
-                                                    int32_t* dstatus, Nodes nd) {
-  __shared__ CtaAppend sh;
-  const int64_t nt = *n_dev;
-  // CTA-uniform passes: every thread reaches the appends
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < nt;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    bool keep = false;
-    if (i < nt) {
-      const uint32_t n0 = resolve_walk(T.s, T.s[i].ra, 2 * nt, dstatus);
-      const uint32_t n1 = resolve_walk(T.s, T.s[i].rb, 2 * nt, dstatus);
-      if (n0 != n1) {
-        T.s[i].na = n0;
-        T.s[i].nb = n1;
-        T.s[i].ra = n0;
-        T.s[i].rb = n1;
-        const unsigned long long tv = (1ull << 44) | (kMask44 - T.s[i].w);
-        if (n0 != nd.immortal) atomicMax(nd.best + n0, tv);
-        if (n1 != nd.immortal) atomicMax(nd.best + n1, tv);
-        keep = true;
-      }
-    }
-    cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
-  }
+  brick0[ft.n] = acc;
 }
 
 // the saddles still live after the rounds, finished in increasing weight in
@@ -2015,12 +1993,13 @@ size_t diagram_batch_workspace_bytes(int64_t nfields, const int64_t* caps, int64
   const int64_t nsad = std::max<int64_t>(std::max<int64_t>(caps[1], caps[2]), 1);
   c.take<unsigned long long>(2 * (nfields + 1));
   c.take<unsigned long long>(look_words(nsad));
+  c.take<int64_t>(nfields + 1);
   return c.used;
 }
 
 int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* desc,
-                         const uint64_t* rec, const dms_field_desc* fields_dev, int nfields,
-                         int64_t total_vertices, int64_t* const crit[4], const int64_t* cnt_dev,
+                         const uint64_t* rec, const dms_field_desc* fields_host,
+                         const dms_field_desc* fields_dev, int nfields, int64_t total_vertices, int64_t* const crit[4], const int64_t* cnt_dev,
                          const int64_t* caps, dms_pair* d0, dms_pair* d2, int64_t cap_pairs,
                          int64_t* pair_offsets, dms_pair* ess, int64_t* pair_totals, void* ws,
                          int32_t* dstatus, cudaStream_t s) {
@@ -2030,6 +2009,7 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   const int64_t nsad = std::max<int64_t>(std::max<int64_t>(caps[1], caps[2]), 1);
   unsigned long long* fcount = c.take<unsigned long long>(2 * (nfields + 1));
   unsigned long long* look = c.take<unsigned long long>(look_words(nsad));
+  int64_t* brick0 = c.take<int64_t>(nfields + 1);
   const FieldTab ft{fields_dev, nfields};
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
@@ -2049,7 +2029,7 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
     unsigned int round = 1;
     for (; large && round <= kBatchLarge; ++round) {
       mem_ok = mem_ok && cudaMemsetAsync(nxt_n, 0, sizeof(unsigned int), s) == cudaSuccess;
-      if (round > 1) {  // b_link_walks did round 1's search
+      if (round > 1) {  // link_d0 / link_d2 did round 1's search
         round_find<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round); count_launch();
       }
       boruvka_hook<<<G, TB, 0, s>>>(cur, cur_n, T, w.nd, round, nxt, nxt_n, w.forest,
@@ -2123,30 +2103,32 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   b_init_nodes_d0<<<G, TB, 0, s>>>(order, crit[0], cnt_dev, w.nd); count_launch();
   b_essential<<<G, TB, 0, s>>>(ft, f, order, crit[0], cnt_dev, ess); count_launch();
-  DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, total_vertices * sizeof(uint32_t), s));
-  mark_ends<<<G, TB, 0, s>>>(crit[0], cnt_dev + 0, 0, 0, w.claim); count_launch();
-  b_d0_weights<<<G, TB, 0, s>>>(ft, order, crit[1], cnt_dev, w.T0); count_launch();
-  {
-    const DescWalk<ManyFields> wk{ManyFields{fields_dev, nfields}, crit[1], desc, w.claim};
-    DMS_TRY(launch_walks(wk, cnt_dev + 1, 0, w.ctr + kCtrWalk, w.T0, dstatus, s));
+  using Desc = DescPaths<ManyFields>;
+  using Dual = DualPaths<ManyFields>;
+  int64_t bricks0 = 0, bricks2 = 0;
+  for (int i = 0; i < nfields; ++i) {
+    bricks0 += brick_count<Desc>(fields_host[i].nx, fields_host[i].ny, fields_host[i].nz);
+    bricks2 += brick_count<Dual>(fields_host[i].nx, fields_host[i].ny, fields_host[i].nz);
   }
+  const ManyFields mf{fields_dev, nfields, brick0};
+  brick_table<<<1, 32, 0, s>>>(ft, Desc::LX, Desc::LY, Desc::LZ, brick0); count_launch();
+  mark_ends<<<G, TB, 0, s>>>(crit[0], cnt_dev + 0, 0, 0, w.path); count_launch();
+  resolve_paths<<<(unsigned)bricks0, kBrickThreads, 0, s>>>(Desc{mf, desc, crit[0], cnt_dev + 0, 0}, w.path); count_launch();
   w.nd.immortal = kNone;
-  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 1, w.T0, w.live0, w.ctr + kCtrLive, dstatus, w.nd); count_launch();
+  link_d0<<<G, TB, 0, s>>>(mf, order, crit[1], cnt_dev + 1, 0, w.path, w.T0, w.live0, w.ctr + kCtrLive,
+                           dstatus, true, w.nd); count_launch();
   DMS_TRY(rounds(w.T0, cnt_dev + 0, 0));
   DMS_TRY(write(0, w.T0, crit[0], crit[1], cnt_dev + 1, d0, pair_offsets, pair_totals + 0, fcount));
 
   // ---- D2
   DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   b_init_nodes_d2<<<G, TB, 0, s>>>(ft, order, crit[3], cnt_dev, w.nd); count_launch();
-  DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, w.nclaim * sizeof(uint32_t), s));
-  mark_ends<<<G, TB, 0, s>>>(crit[3], cnt_dev + 3, 0, 1, w.claim); count_launch();
-  b_d2_weights<<<G, TB, 0, s>>>(ft, order, crit[2], cnt_dev, w.T2); count_launch();
-  {
-    const DualWalk<ManyFields> wk{ManyFields{fields_dev, nfields}, crit[2], rec, w.claim};
-    DMS_TRY(launch_walks(wk, cnt_dev + 2, 0, w.ctr + kCtrWalk, w.T2, dstatus, s));
-  }
+  mark_ends<<<G, TB, 0, s>>>(crit[3], cnt_dev + 3, 0, 1, w.path); count_launch();
+  brick_table<<<1, 32, 0, s>>>(ft, Dual::LX, Dual::LY, Dual::LZ, brick0); count_launch();
+  resolve_paths<<<(unsigned)bricks2, kBrickThreads, 0, s>>>(Dual{mf, rec, crit[3], cnt_dev + 3, 0}, w.path); count_launch();
   w.nd.immortal = 0;  // OUTSIDE, shared by all fields
-  b_link_walks<<<G, TB, 0, s>>>(cnt_dev + 2, w.T2, w.live0, w.ctr + kCtrLive, dstatus, w.nd); count_launch();
+  link_d2<<<G, TB, 0, s>>>(mf, order, crit[2], cnt_dev + 2, 0, w.path, w.T2, w.live0, w.ctr + kCtrLive,
+                           dstatus, true, w.nd); count_launch();
   DMS_TRY(rounds(w.T2, cnt_dev + 3, 1));
   DMS_TRY(write(2, w.T2, crit[2], crit[3], cnt_dev + 2, d2, pair_offsets + (nfields + 1), pair_totals + 1,
                 fcount + (nfields + 1)));
@@ -2211,36 +2193,6 @@ __device__ __forceinline__ uint32_t local_rank2d(const Grid2d& g, const uint32_t
   return r;
 }
 
-__global__ void d0_weights2d(Grid2d g, const uint32_t* __restrict__ order,
-                             const int64_t* __restrict__ crit1, int64_t ne, Tri T) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= ne) return;
-  const int64_t id = crit1[i];
-  const int64_t a = id / 3;
-  const int k = (int)(id - a * 3);
-  const int64_t b = a + cdelta2(g, k + 1);
-  const uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
-  const int64_t top = oa > ob ? a : b;
-  T.s[i].w = ((uint64_t)(oa > ob ? oa : ob) << 4) | local_rank2d(g, order, top, oa > ob ? ob : oa);
-  T.s[i].res = kNone;
-  T.s[i].ra = T.s[i].rb = kNone;  // walk results pending
-  T.s[i].pad = 0;
-}
-
-// D1 saddles are visited by decreasing edge key: D0's weight, complemented
-__global__ void d1_weights2d(int64_t ne, Tri T) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= ne) return;
-  Sad s = T.s[i];
-  s.w = kMask44 - s.w;
-  // On a 2D grid (a disk, no 1-cycles survive) every critical edge is either
-  // a D0 death or a D1 birth: the edges D0 paired take no part in D1.
-  s.pad = s.res != kNone ? 1u : 0u;
-  s.res = kNone;
-  s.ra = s.rb = kNone;  // walk results pending
-  T.s[i] = s;
-}
-
 // node 0 = OUTSIDE (age 0, the oldest); node j + 1 = maximum crit2[j], a
 // higher one older
 __global__ void init_nodes_d1_2d(Grid2d g, const uint32_t* __restrict__ order,
@@ -2272,135 +2224,123 @@ __global__ void init_nodes_d1_2d(Grid2d g, const uint32_t* __restrict__ order,
   nd.age[i] = (kMask44 - key) + 1;
 }
 
-// D0 walks: down the vertex-edge pairs (desc) to a minimum
-struct DescWalk2d {
-  Grid2d g;
-  const int64_t* crit1;
+// D0: down the vertex-edge pairs (desc) to a minimum
+struct DescPaths2d {
+  static constexpr int K = 1, LX = 5, LY = 5, LZ = 0;
+  OneField fields;
   const uint8_t* desc;
-  uint32_t* claim;
-  struct State {
-    int64_t v, it;
-  };
-  __device__ __forceinline__ bool start(int64_t s, int j, State& st, uint32_t&) const {
-    const int64_t id = crit1[s];
-    const int64_t a = id / 3;
-    const int k = (int)(id - a * 3);
-    st.v = j ? a + cdelta2(g, k + 1) : a;
-    st.it = 0;
-    return true;
-  }
-  __device__ __forceinline__ bool step(State& st, uint32_t w, uint32_t& r,
-                                       int32_t* dstatus) const {
-    const uint8_t d = __ldg(desc + st.v);
-    const uint32_t old = atomicCAS(claim + st.v, kUnclaimed, w);
-    if (old != kUnclaimed) {
-      r = claim_result(old);
-      return false;
+  const int64_t* ends;
+  int64_t n;
+  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
+                                        int y0, int, bool, uint32_t (&w)[K]) const {
+    const int d = __ldg(desc + v);
+    if (d >= 6) {
+      if (d == 15) w[0] = end_word(path, v, ends, n, 0);
+      return;
     }
-    if (d >= 6) {  // a minimum without its end mark: inconsistent input
-      set_status(dstatus, DMS_ERR_ARG);
-      r = 0;
-      return false;
-    }
-    st.v += slot_delta2(g, d);
-    if (++st.it > g.n) {
-      set_status(dstatus, DMS_ERR_TIMEOUT);
-      r = 0;
-      return false;
-    }
-    return true;
+    const int c = corner2(d), s = d < 3 ? 1 : -1;
+    const uint32_t to = packed_coords<DescPaths2d>(lv) + s * packed_step(c & 1, (c >> 1) & 1, 0);
+    const bool in = inside<DescPaths2d>(to, x0, y0, 0, (uint32_t)g.nx, (uint32_t)g.ny, 1u);
+    if (in) w[0] = brick_word<DescPaths2d>(to, 0);  // (outside: bad data)
   }
 };
 
-// D1 walks: from a triangle through the edge it is paired with to that
-// edge's other triangle, up to a maximum (node j + 1) or out of the grid
-// (OUTSIDE, node 0).  Claims are indexed by triangle id.
-struct DualWalk2d {
-  Grid2d g;
-  const int64_t* crit1;
+// D1: from a triangle through the edge it is paired with to that edge's other
+// triangle, up to a maximum (node j + 1) or out of the grid (OUTSIDE, node 0)
+struct DualPaths2d {
+  static constexpr int K = 2, LX = 5, LY = 5, LZ = 0;
+  OneField fields;
   const uint16_t* rec;
-  uint32_t* claim;
-  struct State {
-    int64_t b, bx, by, it;
-    int k;
-  };
-  // triangle j of edge id's two (0 or 1), -1 if that square is outside
-  __device__ __forceinline__ bool start(int64_t s, int j, State& st, uint32_t& r) const {
-    const int64_t id = crit1[s];
-    const int64_t a = id / 3;
-    const int t = (int)(id - a * 3);
-    int64_t ax, ay;
-    xy2(g, a, ax, ay);
-    int64_t bx = ax, by = ay;
-    int k;
-    if (t == 2) {
-      k = j;  // both triangles of the square anchored at a
-    } else if (j == 0) {
-      k = t;  // horizontal: the square above, type 0; vertical: the square to the right, type 1
-    } else {
-      if (t == 0) by -= 1;  // horizontal: the square below, type 1
-      else bx -= 1;         // vertical: the square to the left, type 0
-      k = 1 - t;
-    }
-    if (!square2(g, bx, by)) {
-      r = 0;
-      return false;
-    }
-    st.bx = bx;
-    st.by = by;
-    st.b = bx + g.nx * by;
-    st.k = k;
-    st.it = 0;
-    return true;
-  }
-  __device__ __forceinline__ bool step(State& st, uint32_t w, uint32_t& r,
-                                       int32_t* dstatus) const {
-    const uint32_t rw = __ldg(rec + st.b);
-    const uint32_t old = atomicCAS(claim + st.b * 2 + st.k, kUnclaimed, w);
-    if (old != kUnclaimed) {
-      r = claim_result(old);
-      return false;
-    }
-    const uint32_t code = (rw >> (9 + 3 * st.k)) & 7u;
-    if (code < 1u || code > 3u) {  // a critical triangle without its end mark, or bad data
-      set_status(dstatus, DMS_ERR_ARG);
-      r = 0;
-      return false;
-    }
-    // the paired facet and the triangle across it
-    const int om = (int)code - 1;
-    if (om == 1) {
-      st.k = 1 - st.k;  // the diagonal: the other triangle of the square
-    } else if (st.k == 0) {
-      if (om == 0) {  // vertical edge at b + x: the square to the right
-        st.bx += 1;
-        st.k = 1;
-      } else {  // horizontal edge at b: the square below
-        st.by -= 1;
-        st.k = 1;
-      }
-    } else {
-      if (om == 0) {  // horizontal edge at b + y: the square above
-        st.by += 1;
-        st.k = 0;
-      } else {  // vertical edge at b: the square to the left
-        st.bx -= 1;
-        st.k = 0;
+  const int64_t* ends;
+  int64_t n;
+  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
+                                        int y0, int, bool, uint32_t (&w)[K]) const {
+    const uint32_t rw = __ldg(rec + v), at = packed_coords<DualPaths2d>(lv);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t code = (rw >> (9 + 3 * k)) & 7u;
+      if (code == 7u) {
+        w[k] = end_word(path, v * 2 + k, ends, n, 1);
+      } else if (code >= 1u && code <= 3u) {  // (else no triangle there, or bad data)
+        // across the facet that omits chain vertex code - 1: the diagonal
+        // (code 2): the square's other triangle; type 0 (code 1 / 3): the
+        // square to the right / below; type 1: above / to the left
+        const uint32_t to = at + (code == 2u ? 0u : (code == 1u ? (k == 0 ? packed_step(1, 0, 0) : packed_step(0, 1, 0))
+                                                          : (k == 0 ? packed_step(0, -1, 0) : packed_step(-1, 0, 0))));
+        const bool in = inside<DualPaths2d>(to, x0, y0, 0, (uint32_t)(g.nx - 1), (uint32_t)(g.ny - 1), 1u);
+        w[k] = in ? brick_word<DualPaths2d>(to, 1 - k) : kEnd;
       }
     }
-    if (!square2(g, st.bx, st.by)) {
-      r = 0;  // OUTSIDE
-      return false;
-    }
-    st.b = st.bx + g.nx * st.by;
-    if (++st.it > 2 * g.n) {
-      set_status(dstatus, DMS_ERR_TIMEOUT);
-      r = 0;
-      return false;
-    }
-    return true;
   }
 };
+
+__host__ __device__ __forceinline__ Grid grid_of2d(const Grid2d& g) { return Grid{g.nx, g.ny, 1, g.n, g.n}; }
+
+// D0: each critical edge's weight, its two descending paths
+__global__ void __launch_bounds__(256) link2d_d0(Grid2d g, const uint32_t* __restrict__ order,
+                                                 const int64_t* __restrict__ crit1, int64_t ne,
+                                                 const uint32_t* __restrict__ path, Tri T,
+                                                 uint32_t* live, unsigned int* live_n,
+                                                 int32_t* dstatus, Nodes nd) {
+  __shared__ CtaAppend sh;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool keep = false;
+  if (i < ne) {
+    const int64_t id = crit1[i], a = id / 3;
+    const int c = (int)(id - a * 3) + 1;
+    const int64_t b = a + cdelta2(g, c);
+    const Grid g3 = grid_of2d(g);
+    int64_t x, y;
+    xy2(g, a, x, y);
+    Walk wa = walk_from<DescPaths2d>(path, g3, a, (int)x, (int)y, 0, 0);
+    Walk wb = walk_from<DescPaths2d>(path, g3, b, (int)x + (c & 1), (int)y + ((c >> 1) & 1), 0, 0);
+    const uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
+    const uint64_t w = ((uint64_t)(oa > ob ? oa : ob) << 4) |
+                       local_rank2d(g, order, oa > ob ? a : b, oa > ob ? ob : oa);
+    walk_both<DescPaths2d>(path, g3, 0, wa, wb);
+    keep = store_saddle(T, i, w, walk_end(wa, dstatus), walk_end(wb, dstatus), false, nd);
+  }
+  cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+}
+
+// D1: saddles are visited by decreasing edge key (D0's weight, complemented),
+// two dual paths each.  On a 2D grid (a disk, no 1-cycles survive) every
+// critical edge is either a D0 death or a D1 birth: the edges that D0 paired
+// take no part.
+__global__ void __launch_bounds__(256) link2d_d1(Grid2d g, const int64_t* __restrict__ crit1, int64_t ne,
+                                                 const uint32_t* __restrict__ path, Tri T,
+                                                 uint32_t* live, unsigned int* live_n,
+                                                 int32_t* dstatus, Nodes nd) {
+  __shared__ CtaAppend sh;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool keep = false;
+  if (i < ne) {
+    if (T.s[i].res != kNone) {
+      T.s[i].res = kNone;
+    } else {
+      const int64_t id = crit1[i], a = id / 3;
+      const int t = (int)(id - a * 3);
+      const Grid g3 = grid_of2d(g);
+      int64_t ax, ay;
+      xy2(g, a, ax, ay);
+      Walk wk[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        // triangle j of the edge: the diagonal's are both in the square at a;
+        // a horizontal edge's: type 0 above, type 1 below; a vertical edge's:
+        // type 1 to the right, type 0 to the left
+        const int64_t bx = ax - (j == 1 && t == 1), by = ay - (j == 1 && t == 0);
+        const int k = t == 2 ? j : (j == 0 ? t : 1 - t);
+        wk[j] = square2(g, bx, by) ? walk_from<DualPaths2d>(path, g3, bx + g.nx * by, (int)bx, (int)by, 0, k)
+                                   : Walk{kEnd, 0, 0, 0};
+      }
+      walk_both<DualPaths2d>(path, g3, 0, wk[0], wk[1]);
+      keep = store_saddle(T, i, kMask44 - T.s[i].w, walk_end(wk[0], dstatus), walk_end(wk[1], dstatus),
+                          false, nd);
+    }
+  }
+  cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+}
 
 __device__ __forceinline__ int64_t top2(const uint32_t* order, const int64_t* v, int m) {
   int64_t best = v[0];
@@ -2504,12 +2444,11 @@ int launch_diagram2d(const float* f, const uint32_t* order, const uint8_t* desc,
   init_nodes_d0<<<nb(nc[0]), TB, 0, s>>>(order, crit0, nc[0], w.nd); count_launch();
   write_essential<<<nb(nc[0]), TB, 0, s>>>(f, order, crit0, nc[0], ess); count_launch();
   if (ne > 0) {
-    DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, g.n * sizeof(uint32_t), s));
-    mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.claim); count_launch();
-    d0_weights2d<<<nb(ne), TB, 0, s>>>(g, order, crit1, ne, w.T0); count_launch();
-    const DescWalk2d wk{g, crit1, desc, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + kCtrWalk, w.T0, dstatus, s));
-    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + kCtrLive, dstatus); count_launch();
+    mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.path); count_launch();
+    resolve_paths<<<(unsigned)brick_count<DescPaths2d>(nx, ny, 1), kBrickThreads, 0, s>>>(
+        DescPaths2d{OneField{grid_of2d(g)}, desc, crit0, nc[0]}, w.path); count_launch();
+    link2d_d0<<<nb(ne), TB, 0, s>>>(g, order, crit1, ne, w.path, w.T0, w.live0, w.ctr + kCtrLive, dstatus,
+                                    w.nd); count_launch();
   }
   w.nd.immortal = kNone;
   int st = run_pairing(w, w.T0, ne, nc[0], s, dstatus, false);
@@ -2521,14 +2460,13 @@ int launch_diagram2d(const float* f, const uint32_t* order, const uint8_t* desc,
   DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
   init_nodes_d1_2d<<<nb(nc[2] + 1), TB, 0, s>>>(g, order, crit2, nc[2], w.nd); count_launch();
   if (ne > 0) {
-    DMS_CUDA_OK(cudaMemsetAsync(w.claim, 0xFF, 2 * g.n * sizeof(uint32_t), s));
     if (nc[2] > 0) {
-      mark_ends<<<nb(nc[2]), TB, 0, s>>>(crit2, nullptr, nc[2], 1, w.claim); count_launch();
+      mark_ends<<<nb(nc[2]), TB, 0, s>>>(crit2, nullptr, nc[2], 1, w.path); count_launch();
     }
-    d1_weights2d<<<nb(ne), TB, 0, s>>>(ne, w.T0); count_launch();
-    const DualWalk2d wk{g, crit1, rec, w.claim};
-    DMS_TRY(launch_walks(wk, nullptr, ne, w.ctr + kCtrWalk, w.T0, dstatus, s));
-    link_walks<<<nb(ne), TB, 0, s>>>(ne, w.T0, w.live0, w.ctr + kCtrLive, dstatus, true); count_launch();
+    resolve_paths<<<(unsigned)brick_count<DualPaths2d>(nx, ny, 1), kBrickThreads, 0, s>>>(
+        DualPaths2d{OneField{grid_of2d(g)}, rec, crit2, nc[2]}, w.path); count_launch();
+    link2d_d1<<<nb(ne), TB, 0, s>>>(g, crit1, ne, w.path, w.T0, w.live0, w.ctr + kCtrLive, dstatus,
+                                    w.nd); count_launch();
   }
   w.nd.immortal = 0;  // OUTSIDE
   st = run_pairing(w, w.T0, ne, nc[2] + 1, s, dstatus, false);
