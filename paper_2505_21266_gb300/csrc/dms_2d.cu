@@ -4,11 +4,20 @@
 //
 // The triangulation splits every square along its (1,1) diagonal.  A vertex
 // x has six neighbour slots -- s < 3: x + corner, s >= 3: x - corner, corner
-// {+x, +y, +x+y}[s % 3] -- six edges and six triangles around it, in cyclic
-// order T0..T5 below.  ProcessLowerStars runs on 6-bit masks; the records
+// {+x, +y, +x+y}[s % 3] -- six edges and six triangles around it.  The records
 // (rec2, one uint16 per anchor, layout in include/dms.h) are assembled per
 // CTA tile in shared memory from the lower stars of the tile's vertices and
 // a one-vertex halo on the +x and +y sides, then written coalesced.
+//
+// ProcessLowerStars in closed form.  The link of x is a cycle of six vertices,
+// and the lower star is the cone over the arcs of it that precede x.  An arc
+// of n vertices has n edges and n - 1 triangles; popped by key, every triangle
+// pairs with its edge farther from the arc's lowest vertex.  The edge to the
+// lowest vertex of all is paired with x, that of every other arc is critical.
+// Where the whole cycle is lower (a maximum), the six triangles in a row,
+// joined across the edges but the one paired with x, pair with the edges
+// towards the one of largest key, which is critical.  So the lowest vertex of
+// each arc picks a ready-made set of record bits from a table.
 #include <algorithm>
 #include <cstdint>
 
@@ -36,42 +45,74 @@ namespace {
 // at x minus corner {0,0,0,+x,+y,+x+y}[s] (edgeAnc), type s % 3; its two
 // triangles by increasing id on the unbounded lattice are kEdgeCof[s][0..1].
 constexpr int kTriA[6] = {0, 0, 1, 1, 3, 4};
-constexpr int kTriB[6] = {2, 4, 2, 3, 5, 5};
 constexpr int kOmitA[6] = {2, 0, 2, 0, 0, 0};
 constexpr int kOmitB[6] = {1, 2, 1, 2, 1, 1};
 constexpr int kEdgeCof[6][2] = {{1, 0}, {3, 2}, {0, 2}, {4, 3}, {5, 1}, {5, 4}};
 
-struct Star2 {
-  uint8_t triMaskOfSlot[6];  // the two triangles holding edge slot s
-  uint8_t slotsOfTri[6];     // the two slots of triangle j (mask)
-  uint8_t cofIdx[6][6];      // [s][j]: index of triangle j among edge s's triangles
-  uint8_t omit[6][6];        // [j][s]: chain vertex the facet {x, s} of triangle j omits
-};
+constexpr int kTriAnc[6] = {0, 2, 0, 1, 3, 3};   // corner between x and the triangle's anchor
+constexpr int kTriType[6] = {0, 1, 1, 0, 1, 0};
+constexpr int kEdgeAnc[6] = {0, 0, 0, 1, 2, 3};  // the same for the edge of a slot
+// the link's cycle: slots by position; the triangle between positions i, i + 1
+constexpr int kCycSlot[6] = {0, 4, 5, 3, 1, 2};
+constexpr int kCycTri[6] = {1, 5, 4, 3, 2, 0};
 
+// record bits as four 16-bit fields: field c goes to the anchor x - corner c
+constexpr uint64_t edge_bits(int pos, int code) {
+  const int s = kCycSlot[pos];
+  return (uint64_t)code << (16 * kEdgeAnc[s] + 3 * (s % 3));
+}
+constexpr uint64_t tri_bits(int i, int code) {
+  const int j = kCycTri[i];
+  return (uint64_t)code << (16 * kTriAnc[j] + 9 + 3 * kTriType[j]);
+}
+// triangle i (between positions i and i + 1) paired with the edge at pos, one
+// of the two
+constexpr uint64_t pair_bits(int i, int pos) {
+  const int j = kCycTri[i], s = kCycSlot[pos];
+  const int w = kEdgeCof[s][1] == j ? 1 : 0, omit = s == kTriA[j] ? kOmitA[j] : kOmitB[j];
+  return edge_bits(pos, 1 + w) | tri_bits(i, 1 + omit);
+}
+
+struct Star2 {
+  uint64_t arc[64][6];   // [arc][position of its lowest vertex]
+  uint64_t whole[6][6];  // [position of the lowest vertex][the critical triangle]
+  uint64_t crit[6];      // the edge at a position critical
+  uint8_t arc_of[64][8];  // [lower positions][position]: the arc that holds it
+};
 constexpr Star2 make_star2() {
   Star2 t{};
-  for (int j = 0; j < 6; ++j) {
-    t.slotsOfTri[j] = (uint8_t)((1u << kTriA[j]) | (1u << kTriB[j]));
-    t.triMaskOfSlot[kTriA[j]] |= (uint8_t)(1u << j);
-    t.triMaskOfSlot[kTriB[j]] |= (uint8_t)(1u << j);
-    t.omit[j][kTriA[j]] = (uint8_t)kOmitA[j];
-    t.omit[j][kTriB[j]] = (uint8_t)kOmitB[j];
+  for (int L = 0; L < 64; ++L)
+    for (int w = 0; w < 6; ++w) {
+      if (!((L >> w) & 1)) continue;
+      int m = 1 << w;
+      uint64_t e = 0;
+      for (int i = w, k = 0; k < 5 && ((L >> ((i + 1) % 6)) & 1); i = (i + 1) % 6, ++k) {
+        m |= 1 << ((i + 1) % 6);
+        e |= pair_bits(i, (i + 1) % 6);
+      }
+      if (L != 63)
+        for (int i = w; (L >> ((i + 5) % 6)) & 1; i = (i + 5) % 6) {
+          m |= 1 << ((i + 5) % 6);
+          e |= pair_bits((i + 5) % 6, (i + 5) % 6);
+        }
+      t.arc_of[L][w] = (uint8_t)m;
+      if (m == L && L != 63) t.arc[L][w] = e;
+    }
+  for (int w = 0; w < 6; ++w) {
+    t.crit[w] = edge_bits(w, 7);
+    for (int r = 0; r < 6; ++r) {  // triangles w, w + 1, .. in a row, r the critical one
+      uint64_t e = tri_bits(r, 7);
+      for (int i = w; i != r; i = (i + 1) % 6) e |= pair_bits(i, (i + 1) % 6);
+      for (int i = (w + 5) % 6; i != r; i = (i + 5) % 6) e |= pair_bits(i, i);
+      t.whole[w][r] = e;
+    }
   }
-  for (int s = 0; s < 6; ++s)
-    for (int w = 0; w < 2; ++w) t.cofIdx[s][kEdgeCof[s][w]] = (uint8_t)w;
   return t;
 }
-__constant__ Star2 cStar2 = make_star2();
+__device__ const Star2 cStar2 = make_star2();
 
-// the same tables as 4-bit fields of immediates, for indices known only at
-// run time in device code
-__device__ __forceinline__ int triA(int j) { return (0x431100 >> (4 * j)) & 15; }
-__device__ __forceinline__ int triB(int j) { return (0x553242 >> (4 * j)) & 15; }
-__device__ __forceinline__ int triAnc(int j) { return (0x331020 >> (4 * j)) & 15; }
-__device__ __forceinline__ int triType(int j) { return (0x010110 >> (4 * j)) & 15; }
-__device__ __forceinline__ int edgeAnc(int s) { return (0x321000 >> (4 * s)) & 15; }
-
-constexpr int TX2 = 64, TY2 = 16, NT2 = 256;
+// 64 x 16 anchors a CTA, their vertices with the halo in four rounds
+constexpr int TX2 = 64, TY2 = 16, NT2 = 288;
 constexpr int WX2 = TX2 + 3, WY2 = TY2 + 3;
 
 struct Smem2 {
@@ -80,117 +121,78 @@ struct Smem2 {
   uint32_t rec[TY2][TX2];  // records of the tile's anchors
 };
 
-// slot offsets (dx, dy) and anchor corners as bit masks of (+x, +y)
-__device__ __forceinline__ int sdx(int s) { return s < 3 ? ((s + 1) & 1) : -(((s - 3) + 1) & 1); }
-__device__ __forceinline__ int sdy(int s) {
-  return s < 3 ? (((s + 1) >> 1) & 1) : -((((s - 3) + 1) >> 1) & 1);
-}
+// slot offsets (dx, dy)
+constexpr int sdx(int s) { return s < 3 ? ((s + 1) & 1) : -(((s - 3) + 1) & 1); }
+constexpr int sdy(int s) { return s < 3 ? (((s + 1) >> 1) & 1) : -((((s - 3) + 1) >> 1) & 1); }
 
-// ProcessLowerStars of one vertex (the reading of the 3D kernel): returns
-// desc (slot of the paired edge, 15 for a minimum) and the record bits for
-// the four anchors x - corner c in acc[c].
+// the lower star of a vertex of order ox, o[i] the order at position i of its
+// link's cycle: desc (15 for a minimum) and its record bits
 __device__ __forceinline__ int lower_star2(uint32_t ox, const uint32_t (&o)[6], const Star2& tb,
-                                           uint32_t (&acc)[4]) {
+                                           uint64_t& bits) {
+  uint32_t L = 0, lo = 0xFFFFFFFFu;
+  int w = 0;
 #pragma unroll
-  for (int c = 0; c < 4; ++c) acc[c] = 0;
-  uint32_t lm = 0;
-#pragma unroll
-  for (int s = 0; s < 6; ++s) lm |= (o[s] < ox ? 1u : 0u) << s;
-  if (!lm) return 15;
-  uint32_t r[6];
-  int delta = 0;
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    uint32_t k = 0;
-#pragma unroll
-    for (int t = 0; t < 6; ++t)
-      if (t != s) k += ((lm >> t) & 1) && o[t] < o[s] ? 1u : 0u;
-    r[s] = k;
-    if (((lm >> s) & 1) && k == 0) delta = s;
-  }
-  uint32_t TL = 0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j)
-    if ((tb.slotsOfTri[j] & lm) == tb.slotsOfTri[j]) TL |= 1u << j;
-  auto tkey = [&](int j) {
-    const uint32_t a = r[triA(j)], b = r[triB(j)];
-    return ((max(a, b) + 1) << 8) | ((min(a, b) + 1) << 4);
-  };
-  uint32_t cE = 1u << delta, cT = 0, zE = lm & ~cE, zT = 0, pT = 0;
-  uint32_t ecode[6] = {0, 0, 0, 0, 0, 0}, tcode[6] = {0, 0, 0, 0, 0, 0};
-  auto push = [&](int s) {  // triangles of edge s left with one unclassified edge
-    for (uint32_t m = tb.triMaskOfSlot[s] & TL & ~cT; m; m &= m - 1) {
-      const int j = __ffs(m) - 1;
-      if (__popc(tb.slotsOfTri[j] & ~cE) == 1) pT |= 1u << j;
-    }
-  };
-  push(delta);
-  for (int guard = 0; guard < 64; ++guard) {  // at most 12 pushes + 11 pops happen
-    if (pT) {
-      int jb = 0;
-      uint32_t kb = 0xFFFFu;
-      for (uint32_t m = pT; m; m &= m - 1) {
-        const int j = __ffs(m) - 1;
-        const uint32_t k = tkey(j);
-        if (k < kb) { kb = k; jb = j; }
-      }
-      pT &= ~(1u << jb);
-      if ((cT >> jb) & 1) continue;
-      const uint32_t nu = tb.slotsOfTri[jb] & ~cE;
-      if (!nu) {
-        zT |= 1u << jb;
-        continue;
-      }
-      const int beta = __ffs(nu) - 1;
-      ecode[beta] = 1u + tb.cofIdx[beta][jb];
-      tcode[jb] = 1u + tb.omit[jb][beta];
-      cE |= 1u << beta;
-      cT |= 1u << jb;
-      zE &= ~(1u << beta);
-      push(beta);
-      continue;
-    }
-    if (!(zE | zT)) break;
-    uint32_t kb = 0xFFFFu;
-    int ib = 0, isTri = 0;
-    for (uint32_t m = zE; m; m &= m - 1) {
-      const int s = __ffs(m) - 1;
-      const uint32_t k = (r[s] + 1) << 8;
-      if (k < kb) { kb = k; ib = s; isTri = 0; }
-    }
-    for (uint32_t m = zT; m; m &= m - 1) {
-      const int j = __ffs(m) - 1;
-      const uint32_t k = tkey(j);
-      if (k < kb) { kb = k; ib = j; isTri = 1; }
-    }
-    if (isTri) {
-      tcode[ib] = 7;
-      cT |= 1u << ib;
-      zT &= ~(1u << ib);
-    } else {
-      ecode[ib] = 7;
-      cE |= 1u << ib;
-      zE &= ~(1u << ib);
-      push(ib);
+  for (int i = 0; i < 6; ++i) {
+    L |= (o[i] < ox ? 1u : 0u) << i;
+    if (o[i] < lo) {
+      lo = o[i];
+      w = i;
     }
   }
+  bits = 0;
+  if (!L) return 15;
+  if (L == 63u) {
+    // the triangle of largest key: on the highest vertex and the higher of
+    // the two next to it
+    uint32_t hi = 0;
+    int h = 0;
 #pragma unroll
-  for (int s = 0; s < 6; ++s)
-    if ((lm >> s) & 1) acc[edgeAnc(s)] |= ecode[s] << (3 * (s % 3));
+    for (int i = 0; i < 6; ++i)
+      if (o[i] >= hi) {
+        hi = o[i];
+        h = i;
+      }
+    uint32_t next = 0, prev = 0;
 #pragma unroll
-  for (int j = 0; j < 6; ++j)
-    if ((TL >> j) & 1) acc[triAnc(j)] |= tcode[j] << (9 + 3 * triType(j));
-  return delta;
+    for (int i = 0; i < 6; ++i) {
+      next = h == i ? o[(i + 1) % 6] : next;
+      prev = h == i ? o[(i + 5) % 6] : prev;
+    }
+    bits = tb.whole[w][next > prev ? h : (h ? h - 1 : 5)];
+  } else {
+    uint32_t A = tb.arc_of[L][w];
+    bits = tb.arc[A][w];
+    for (uint32_t left = L & ~A; left;) {  // at most two more arcs
+      uint32_t best = 0xFFFFFFFFu;
+      int v = 0;
+#pragma unroll
+      for (int i = 0; i < 6; ++i)
+        if (((left >> i) & 1) && o[i] < best) {
+          best = o[i];
+          v = i;
+        }
+      A = tb.arc_of[left][v];
+      bits |= tb.arc[A][v] | tb.crit[v];
+      left &= ~A;
+    }
+  }
+  return (0x213540 >> (4 * w)) & 15;  // its slot
 }
 
+// Bound by instruction issue (7 bytes of DRAM per vertex are 0.3 ms at 16384^2):
+// the six comparisons, the lowest of them, and where lanes differ the second
+// and third arcs.  With the queues of ProcessLowerStars simulated per vertex
+// it took 13.8 ms at 16384^2 and takes 3.2; 288 threads cover the 65 x 17
+// vertices of a tile in four rounds (256 threads: five).
 __global__ void __launch_bounds__(NT2) gradient2d_kernel(const uint32_t* __restrict__ order,
                                                          int64_t nx, int64_t ny,
                                                          uint8_t* __restrict__ desc,
                                                          uint16_t* __restrict__ rec) {
   __shared__ Smem2 sm;
   const int64_t x0 = (int64_t)blockIdx.x * TX2, y0 = (int64_t)blockIdx.y * TY2;
-  if (threadIdx.x < sizeof(Star2))
-    reinterpret_cast<uint8_t*>(&sm.st)[threadIdx.x] = reinterpret_cast<const uint8_t*>(&cStar2)[threadIdx.x];
+  static_assert(sizeof(Star2) % 8 == 0, "word copy");
+  for (int i = threadIdx.x; i < (int)(sizeof(Star2) / 8); i += NT2)
+    reinterpret_cast<uint64_t*>(&sm.st)[i] = __ldg(reinterpret_cast<const uint64_t*>(&cStar2) + i);
   for (int i = threadIdx.x; i < WX2 * WY2; i += NT2) {
     const int wx = i % WX2, wy = i / WX2;
     const int64_t gx = x0 - 1 + wx, gy = y0 - 1 + wy;
@@ -206,14 +208,18 @@ __global__ void __launch_bounds__(NT2) gradient2d_kernel(const uint32_t* __restr
     const uint32_t ox = sm.win[ly + 1][lx + 1];
     uint32_t o[6];
 #pragma unroll
-    for (int s = 0; s < 6; ++s) o[s] = sm.win[ly + 1 + sdy(s)][lx + 1 + sdx(s)];
-    uint32_t acc[4];
-    const int d = lower_star2(ox, o, sm.st, acc);
+    for (int c = 0; c < 6; ++c) {
+      constexpr int slots[6] = {0, 4, 5, 3, 1, 2};
+      o[c] = sm.win[ly + 1 + sdy(slots[c])][lx + 1 + sdx(slots[c])];
+    }
+    uint64_t bits;
+    const int d = lower_star2(ox, o, sm.st, bits);
     if (lx < TX2 && ly < TY2) desc[gx + nx * gy] = (uint8_t)d;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int ax = lx - (c & 1), ay = ly - ((c >> 1) & 1);
-      if (acc[c] && ax >= 0 && ay >= 0 && ax < TX2 && ay < TY2) atomicOr(&sm.rec[ay][ax], acc[c]);
+      const uint32_t m = (uint32_t)(bits >> (16 * c)) & 0xFFFFu;
+      if (m && ax >= 0 && ay >= 0 && ax < TX2 && ay < TY2) atomicOr(&sm.rec[ay][ax], m);
     }
   }
   __syncthreads();
