@@ -3,16 +3,18 @@
 // sort of the vertices by f, with -0.0 == +0.0 and ties left in offset order.
 //
 // A stable least-significant-digit radix sort of 32-bit order-preserving keys
-// with the vertex index as payload, 8-bit digits, reduce-then-scan per pass:
+// with the vertex index as payload, 8-bit digits, one launch per pass:
 //   * one pre-pass counts the four digit histograms of the whole field and
-//     flags NaNs; a tiny plan kernel then skips every pass whose digit is the
-//     same for all vertices (quantised fields: the low mantissa bytes), so the
-//     decision never leaves the device;
-//   * per pass: an upsweep counts digits per tile, a three-kernel exclusive
-//     scan turns the (digit-major) tile counts into output offsets, and a
-//     downsweep ranks the tile stably (the lanes holding the same digit from
-//     ballots on its bits, then popc), stages it in shared memory in digit
-//     order and writes it out;
+//     flags NaNs; a tiny plan kernel turns them into the digits' first
+//     positions and skips every pass whose digit is the same for all vertices
+//     (quantised fields: the low mantissa bytes), so the decision never leaves
+//     the device;
+//   * per pass: a CTA takes a tile by ticket, ranks it stably (the lanes of a
+//     warp holding the same digit from a mask per digit that each of them ors
+//     its bit into), publishes its digit counts, stages the tile in shared
+//     memory in digit order, learns from the tiles before it how many of each
+//     digit precede (decoupled look-back, one digit per thread), and writes
+//     the tile out;
 //   * the first active pass reads the float field itself (payload = index),
 //     the last one scatters order[payload] = position instead of writing keys;
 //   * on a large field (or batch of fields) that scatter -- 4-byte writes to random
@@ -38,9 +40,8 @@ constexpr int SORT_NT = 512;  // 4 CTAs per SM at 32 registers (a few spilled): 
 constexpr int SORT_ITEMS = 8;
 constexpr int SORT_TILE = SORT_NT * SORT_ITEMS;  // 4096
 constexpr int SORT_WARPS = SORT_NT / 32;
-constexpr int SCAN_NT = 1024;
-constexpr int SCAN_ITEMS = 8;
-constexpr int SCAN_CHUNK = SCAN_NT * SCAN_ITEMS;
+constexpr int kLookAhead = 4;           // tiles read at a time when looking back
+constexpr uint32_t kLookPolls = 1u << 22;
 
 enum : int { SRC_FIELD = 0, SRC_A = 1, SRC_B = 2, DST_A = 1, DST_B = 2, DST_ORDER = 3 };
 
@@ -68,6 +69,9 @@ struct Plan {
   int src[kPasses];
   int dst[kPasses];
   int any;
+  int failed;    // a wait of a pass ran out
+  unsigned int base[kPasses][256];  // first position of each digit
+  unsigned int ticket[kPasses];     // tiles taken
   int last_src;  // source of the last active pass (its other buffers are then free)
 };
 
@@ -111,114 +115,8 @@ __global__ void __launch_bounds__(256) hist_all_kernel(const float* __restrict__
     if ((&h[0][0])[i]) atomicAdd(ghist + i, (&h[0][0])[i]);
 }
 
-__global__ void plan_kernel(const unsigned int* __restrict__ ghist, int64_t n, int nfields,
-                            Plan* plan) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int act[kPasses];
-  for (int p = 0; p < 4; ++p) {
-    unsigned int mx = 0;
-    for (int d = 0; d < 256; ++d) mx = max(mx, ghist[p * 256 + d]);
-    act[p] = (int64_t)mx != n;
-  }
-  act[4] = nfields > 1;
-  act[5] = nfields > 256;
-  int last = -1, first = -1, cnt = 0;
-  for (int p = 0; p < kPasses; ++p)
-    if (act[p]) {
-      if (first < 0) first = p;
-      last = p;
-      ++cnt;
-    }
-  int cur = SRC_FIELD, k = 0;
-  plan->last_src = SRC_FIELD;
-  for (int p = 0; p < kPasses; ++p) {
-    plan->active[p] = act[p];
-    plan->src[p] = plan->dst[p] = 0;
-    if (!act[p]) continue;
-    plan->src[p] = cur;
-    plan->last_src = cur;
-    int dst = (p == last) ? DST_ORDER : ((k & 1) ? DST_B : DST_A);
-    plan->dst[p] = dst;
-    cur = dst;
-    ++k;
-  }
-  plan->any = cnt > 0;
-}
-
-__device__ __forceinline__ void load_key(int src, const float* f, const uint32_t* ka,
-                                         const uint32_t* kb, int64_t i, uint32_t& k) {
-  bool nan = false;
-  if (src == SRC_FIELD) k = canon_key(__ldg(f + i), &nan);
-  else k = __ldg((src == SRC_A ? ka : kb) + i);
-}
-
-// digit of pass p: a key byte, or a byte of the vertex's field index
-__device__ __forceinline__ uint32_t digit_of(int pass, uint32_t key, uint32_t val, const Fields& fl) {
-  if (pass < 4) return (key >> (8 * pass)) & 255u;
-  return (field_of(fl, val) >> (8 * (pass - 4))) & 255u;
-}
-
-// per-tile digit counts, digit-major: th[d * ntiles + tile]
-__global__ void __launch_bounds__(SORT_NT) upsweep_kernel(int pass, const Plan* __restrict__ plan,
-                                                          const float* __restrict__ f,
-                                                          const uint32_t* __restrict__ ka,
-                                                          const uint32_t* __restrict__ kb,
-                                                          const uint32_t* __restrict__ va,
-                                                          const uint32_t* __restrict__ vb,
-                                                          const Fields fl, int64_t n,
-                                                          int64_t ntiles,
-                                                          unsigned int* __restrict__ th) {
-  if (!plan->active[pass]) return;
-  const int src = plan->src[pass];
-  __shared__ unsigned int h[SORT_WARPS][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < SORT_WARPS * 256; i += SORT_NT) (&h[0][0])[i] = 0;
-  __syncthreads();
-  const int64_t tile0 = (int64_t)blockIdx.x * SORT_TILE;
-  const uint32_t* kp = src == SRC_FIELD ? reinterpret_cast<const uint32_t*>(f)
-                                        : (src == SRC_A ? ka : kb);
-  if (pass < 4 && tile0 + SORT_TILE <= n && (reinterpret_cast<uintptr_t>(kp) & 15) == 0) {
-    // a whole tile of key bits in 16-byte loads (counts need no order)
-    const uint4* k4 = reinterpret_cast<const uint4*>(kp + tile0);
-    for (int q = threadIdx.x; q < SORT_TILE / 4; q += SORT_NT) {
-      const uint4 w = __ldg(k4 + q);
-      const uint32_t b[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t k = b[j];
-        if (src == SRC_FIELD) {
-          bool nan = false;
-          k = canon_key(__uint_as_float(k), &nan);
-        }
-        atomicAdd(&h[warp][(k >> (8 * pass)) & 255u], 1u);
-      }
-    }
-  } else {
-    const int64_t base = tile0 + (int64_t)warp * (32 * SORT_ITEMS);
-    for (int r = 0; r < SORT_ITEMS; ++r) {
-      int64_t i = base + r * 32 + lane;
-      uint32_t d = 256u + lane;  // unique dummy digit for the ragged tail
-      if (i < n) {
-        uint32_t k = 0, v = (uint32_t)i;
-        if (pass < 4) load_key(src, f, ka, kb, i, k);
-        else if (src != SRC_FIELD) v = __ldg((src == SRC_A ? va : vb) + i);
-        d = digit_of(pass, k, v, fl);
-      }
-      if (d < 256u) atomicAdd(&h[warp][d], 1u);  // counts only: no order needed
-    }
-  }
-  __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += SORT_NT) {
-    unsigned int s = 0;
-    for (int w = 0; w < SORT_WARPS; ++w) s += h[w][d];
-    th[(int64_t)d * ntiles + blockIdx.x] = s;
-  }
-}
-
-// exclusive scan of a uint32 array in three kernels (chunk sums, scan of the
-// sums in one CTA, chunk scans with offsets); skipped for inactive passes
-__device__ __forceinline__ unsigned int block_excl_scan(unsigned int v, unsigned int* tmp,
-                                                        unsigned int* total) {
+// exclusive scan over a CTA's threads
+__device__ __forceinline__ unsigned int block_excl_scan(unsigned int v, unsigned int* tmp) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned int x = v;
 #pragma unroll
@@ -238,136 +136,169 @@ __device__ __forceinline__ unsigned int block_excl_scan(unsigned int v, unsigned
     tmp[lane] = w;  // inclusive warp totals
   }
   __syncthreads();
-  unsigned int excl = x - v + (warp > 0 ? tmp[warp - 1] : 0u);
-  if (total) *total = tmp[(blockDim.x >> 5) - 1];
+  const unsigned int excl = x - v + (warp > 0 ? tmp[warp - 1] : 0u);
   __syncthreads();
   return excl;
 }
 
-__global__ void __launch_bounds__(SCAN_NT) scan_reduce_kernel(int pass, const Plan* plan,
-                                                              const unsigned int* __restrict__ a,
-                                                              int64_t m, unsigned int* sums) {
-  if (plan && !plan->active[pass]) return;
+// one CTA of 256 threads, a digit each
+__global__ void __launch_bounds__(256) plan_kernel(const unsigned int* __restrict__ ghist, int64_t n,
+                                                   const Fields fl, Plan* plan) {
   __shared__ unsigned int tmp[32];
-  const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK;
-  unsigned int s = 0;
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    int64_t i = base + (int64_t)k * SCAN_NT + threadIdx.x;
-    if (i < m) s += a[i];
-  }
-  unsigned int total;
-  block_excl_scan(s, tmp, &total);
-  if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(SCAN_NT) scan_sums_kernel(int pass, const Plan* plan,
-                                                            unsigned int* sums, int64_t nsums) {
-  if (plan && !plan->active[pass]) return;
-  __shared__ unsigned int tmp[32];
-  __shared__ unsigned int carry;
-  if (threadIdx.x == 0) carry = 0;
+  __shared__ unsigned int cnt[2][256];
+  const int d = threadIdx.x;
+  // vertices by the two bytes of their field's index
+  cnt[0][d] = cnt[1][d] = 0;
   __syncthreads();
-  for (int64_t b = 0; b < nsums; b += SCAN_NT) {
-    int64_t i = b + threadIdx.x;
-    unsigned int v = i < nsums ? sums[i] : 0u;
-    unsigned int total;
-    unsigned int e = block_excl_scan(v, tmp, &total);
-    if (i < nsums) sums[i] = e + carry;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += total;
-    __syncthreads();
+  if (fl.n > 1)
+    for (int f = d; f < fl.n; f += 256) {
+      const unsigned int size = (unsigned int)(fl.off[f + 1] - fl.off[f]);
+      atomicAdd(&cnt[0][f & 255], size);
+      atomicAdd(&cnt[1][(f >> 8) & 255], size);
+    }
+  __syncthreads();
+  int act[kPasses];
+#pragma unroll
+  for (int p = 0; p < kPasses; ++p) {
+    const unsigned int c = p < 4 ? ghist[p * 256 + d] : cnt[p - 4][d];
+    plan->base[p][d] = block_excl_scan(c, tmp);
+    act[p] = __syncthreads_or((int64_t)c == n) == 0;
   }
+  act[4] = fl.n > 1;
+  act[5] = fl.n > 256;
+  if (d != 0) return;
+  int last = -1, cnt_act = 0;
+  for (int p = 0; p < kPasses; ++p)
+    if (act[p]) {
+      last = p;
+      ++cnt_act;
+    }
+  int cur = SRC_FIELD, k = 0;
+  plan->last_src = SRC_FIELD;
+  for (int p = 0; p < kPasses; ++p) {
+    plan->active[p] = act[p];
+    plan->src[p] = plan->dst[p] = 0;
+    plan->ticket[p] = 0;
+    if (!act[p]) continue;
+    plan->src[p] = cur;
+    plan->last_src = cur;
+    int dst = (p == last) ? DST_ORDER : ((k & 1) ? DST_B : DST_A);
+    plan->dst[p] = dst;
+    cur = dst;
+    ++k;
+  }
+  plan->any = cnt_act > 0;
+  plan->failed = 0;
 }
 
-__global__ void __launch_bounds__(SCAN_NT) scan_down_kernel(int pass, const Plan* plan,
-                                                            unsigned int* __restrict__ a, int64_t m,
-                                                            const unsigned int* __restrict__ sums) {
-  if (plan && !plan->active[pass]) return;
-  __shared__ unsigned int tmp[32];
-  const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
-  unsigned int v[SCAN_ITEMS];
-  unsigned int s = 0;
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    int64_t i = base + k;
-    v[k] = i < m ? a[i] : 0u;
-    s += v[k];
-  }
-  unsigned int e = block_excl_scan(s, tmp, nullptr) + sums[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    int64_t i = base + k;
-    if (i < m) a[i] = e;
-    e += v[k];
-  }
+__device__ __forceinline__ void load_key(int src, const float* f, const uint32_t* ka,
+                                         const uint32_t* kb, int64_t i, uint32_t& k) {
+  bool nan = false;
+  if (src == SRC_FIELD) k = canon_key(__ldg(f + i), &nan);
+  else k = __ldg((src == SRC_A ? ka : kb) + i);
+}
+
+// digit of pass p: a key byte, or a byte of the vertex's field index
+__device__ __forceinline__ uint32_t digit_of(int pass, uint32_t key, uint32_t val, const Fields& fl) {
+  if (pass < 4) return (key >> (8 * pass)) & 255u;
+  return (field_of(fl, val) >> (8 * (pass - 4))) & 255u;
 }
 
 struct DownSmem {
-  unsigned int wh[SORT_WARPS][256];  // per-warp digit counts, then warp offsets
-  unsigned int dstart[256];          // first local position of each digit
-  unsigned int goff[256];            // global offset of each digit for this tile
+  unsigned int wh[SORT_WARPS][256];  // per-warp digit counts, then where a warp's digits start
+  unsigned int goff[256];            // global minus local position of each digit
   unsigned int tmp[32];
-  uint32_t sk[SORT_TILE];
+  unsigned int tile;
+  union {
+    unsigned int peers[SORT_WARPS][256];  // while ranking: the lanes that hold a digit
+    uint32_t sk[SORT_TILE];               // then: the tile's keys in digit order
+  };
   uint32_t sv[SORT_TILE];
 };
+static_assert(SORT_WARPS * 256 <= SORT_TILE, "the masks fit where the keys go");
 
-__global__ void __launch_bounds__(SORT_NT, 4) downsweep_kernel(
-    int pass, const Plan* __restrict__ plan, const float* __restrict__ f, uint32_t* ka,
-    uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* __restrict__ order, const Fields fl,
-    int64_t n, int64_t ntiles, const unsigned int* __restrict__ th, bool inverse) {
-  if (!plan->active[pass]) return;
+// One pass.  look[tile * 256 + d], zero before the first pass: the tile's count
+// of digit d in bits 0..31, above it 2 * pass + 1 when that is the tile's own
+// count, 2 * pass + 2 when it is the count up to the tile's end.  Tickets are
+// drawn in order, so the tiles that a CTA waits for are running or done; the
+// waits are bounded all the same, and after one that ran out nothing more is
+// sorted.
+// Bound by the shared-memory pipe (78 % of its peak: the masks, the counts,
+// the tile's staging) and by the latency of ranking, with DRAM at a third of
+// its rate.  The whole order took, at 1024^3, 512^3 quantised, 64^3 and 24^3,
+// 52.0, 4.60, 0.254 and 0.225 ms as reduce-then-scan (digit counts per tile,
+// three scan kernels, a second reading of the keys) and takes 44.4, 3.99,
+// 0.18 and 0.15 ms.  Of the tiles, 512 x 12 keys (48.5), 512 x 16 (52.7), 384 x
+// 16 (51.0), 256 x 16 (54.4) and three CTAs per SM (51.9) were slower than 512
+// x 8 in four (47.8), a digit's lanes from eight ballots 49.1; looking back four
+// tiles at a time gave 1.6 ms of it, the offsets in one table 1.8.
+__global__ void __launch_bounds__(SORT_NT, 4) onesweep_kernel(
+    int pass, Plan* __restrict__ plan, const float* __restrict__ f, uint32_t* ka, uint32_t* kb,
+    uint32_t* va, uint32_t* vb, uint32_t* __restrict__ order, const Fields fl, int64_t n,
+    unsigned long long* look, bool inverse, int32_t* dstatus) {
+  if (!plan->active[pass] || plan->failed) return;
   const int src = plan->src[pass], dst = plan->dst[pass];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   DownSmem& sm = *reinterpret_cast<DownSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  for (int i = threadIdx.x; i < SORT_WARPS * 256; i += SORT_NT) (&sm.wh[0][0])[i] = 0;
+  for (int i = threadIdx.x; i < SORT_WARPS * 256; i += SORT_NT) {
+    (&sm.wh[0][0])[i] = 0;
+    (&sm.peers[0][0])[i] = 0;
+  }
+  if (threadIdx.x == 0) sm.tile = atomicAdd(&plan->ticket[pass], 1u);
   __syncthreads();
-  const int64_t tile0 = (int64_t)blockIdx.x * SORT_TILE;
+  const int64_t tile = sm.tile, tile0 = tile * SORT_TILE;
   const int64_t base = tile0 + (int64_t)warp * (32 * SORT_ITEMS);
   uint32_t key[SORT_ITEMS], val[SORT_ITEMS];
   unsigned short pos[SORT_ITEMS];
   const uint32_t* vsrc = src == SRC_A ? va : vb;
+  volatile unsigned int* const peers_of = sm.peers[warp];
+  volatile unsigned int* const count_of = sm.wh[warp];
 #pragma unroll
   for (int r = 0; r < SORT_ITEMS; ++r) {
-    int64_t i = base + r * 32 + lane;
-    uint32_t d = 256u + lane;
+    const int64_t i = base + r * 32 + lane;
+    const bool in = i < n;
+    uint32_t d = 0;
     key[r] = 0;
     val[r] = 0;
-    if (i < n) {
+    if (in) {
       load_key(src, f, ka, kb, i, key[r]);
       val[r] = src == SRC_FIELD ? (uint32_t)i : __ldg(vsrc + i);
       d = digit_of(pass, key[r], val[r], fl);
+      atomicOr(&sm.peers[warp][d], 1u << lane);
     }
-    // lanes with the same digit: eight ballots on its bits and one on validity
-    unsigned peers = __ballot_sync(0xFFFFFFFFu, d < 256u);
-    if (d >= 256u) peers = ~peers;
-#pragma unroll
-    for (int bit = 0; bit < 8; ++bit) {
-      const unsigned bal = __ballot_sync(0xFFFFFFFFu, (d >> bit) & 1u);
-      peers &= ((d >> bit) & 1u) ? bal : ~bal;
-    }
-    unsigned int b = d < 256u ? sm.wh[warp][d] : 0u;
+    __syncwarp();
+    const unsigned peers = in ? peers_of[d] : 0u;
+    const unsigned int b = in ? count_of[d] : 0u;
     __syncwarp();
     pos[r] = (unsigned short)(b + __popc(peers & lt));
-    if (d < 256u && lane == __ffs(peers) - 1) sm.wh[warp][d] = b + __popc(peers);
+    if (in && lane == 31 - __clz(peers)) {  // the last of them
+      count_of[d] = b + __popc(peers);
+      peers_of[d] = 0;
+    }
     __syncwarp();
   }
   __syncthreads();
-  // warp offsets per digit, digit totals, local digit starts, global offsets
+  // warp offsets per digit, digit totals (published), local digit starts
   unsigned int tot = 0;
+  volatile unsigned long long* const mine = look + tile * 256 + threadIdx.x;
+  const unsigned long long own = (unsigned long long)(2 * pass + 1) << 32;
+  const unsigned long long upto = (unsigned long long)(2 * pass + 2) << 32;
   if (threadIdx.x < 256) {
-    const int d = threadIdx.x;
-    for (int w = 0; w < SORT_WARPS; ++w) {
-      unsigned int c = sm.wh[w][d];
-      sm.wh[w][d] = tot;
-      tot += c;
-    }
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) tot += sm.wh[w][threadIdx.x];
+    *mine = (tile == 0 ? upto : own) | tot;
   }
-  unsigned int ds = block_excl_scan(threadIdx.x < 256 ? tot : 0u, sm.tmp, nullptr);
+  const unsigned int ds = block_excl_scan(threadIdx.x < 256 ? tot : 0u, sm.tmp);
   if (threadIdx.x < 256) {
-    sm.dstart[threadIdx.x] = ds;
-    sm.goff[threadIdx.x] = th[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    unsigned int at = ds;
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) {
+      const unsigned int c = sm.wh[w][threadIdx.x];
+      sm.wh[w][threadIdx.x] = at;
+      at += c;
+    }
   }
   __syncthreads();
 #pragma unroll
@@ -375,10 +306,34 @@ __global__ void __launch_bounds__(SORT_NT, 4) downsweep_kernel(
     int64_t i = base + r * 32 + lane;
     if (i < n) {
       uint32_t d = digit_of(pass, key[r], val[r], fl);
-      unsigned int p = sm.dstart[d] + sm.wh[warp][d] + pos[r];
+      unsigned int p = sm.wh[warp][d] + pos[r];
       sm.sk[p] = key[r];
       sm.sv[p] = val[r];
     }
+  }
+  if (threadIdx.x < 256) {
+    unsigned int before = 0;
+    bool done = false;
+    for (int64_t j = tile - 1; j >= 0 && !done; j -= kLookAhead) {
+      unsigned long long v[kLookAhead];
+#pragma unroll
+      for (int q = 0; q < kLookAhead; ++q)
+        v[q] = j >= q ? *(volatile unsigned long long*)(look + (j - q) * 256 + threadIdx.x) : upto;
+#pragma unroll
+      for (int q = 0; q < kLookAhead; ++q) {
+        if (done) continue;
+        volatile unsigned long long* const st = look + (j - q) * 256 + threadIdx.x;
+        for (uint32_t it = 0; v[q] < own && it < kLookPolls; ++it) v[q] = *st;
+        if (v[q] < own) {
+          plan->failed = 1;
+          set_status(dstatus, DMS_ERR_TIMEOUT);
+        }
+        before += (unsigned int)v[q];
+        done = v[q] >= upto || v[q] < own;
+      }
+    }
+    if (tile > 0) *mine = upto | (unsigned int)(before + tot);
+    sm.goff[threadIdx.x] = plan->base[pass][threadIdx.x] + before - ds;
   }
   __syncthreads();
   const int64_t cnt = (n - tile0 < (int64_t)SORT_TILE) ? n - tile0 : (int64_t)SORT_TILE;
@@ -388,7 +343,8 @@ __global__ void __launch_bounds__(SORT_NT, 4) downsweep_kernel(
     uint32_t k = sm.sk[p];
     const uint32_t v = sm.sv[p];
     uint32_t d = digit_of(pass, k, v, fl);
-    uint32_t g = sm.goff[d] + (p - sm.dstart[d]);
+    uint32_t g = sm.goff[d] + p;
+    if (g >= n || v >= n) continue;  // (a wait that ran out)
     if (dst == DST_ORDER && inverse) {
       // the payloads in position order, in the value buffer this pass does
       // not read; the inverse-permutation passes build order[] from them
@@ -423,7 +379,7 @@ __global__ void __launch_bounds__(INV_NT, 4) inv_bucket_kernel(
     const Plan* __restrict__ plan, uint32_t* va, uint32_t* vb, const uint32_t* inV,
     const uint32_t* __restrict__ inP, int64_t n, int shift, int nbins, uint32_t* __restrict__ outV,
     uint32_t* __restrict__ outP, unsigned int* __restrict__ cur) {
-  if (!plan->any) return;
+  if (!plan->any || plan->failed) return;
   __shared__ InvSmem sm;
   if (!inV) inV = plan->last_src == SRC_A ? vb : va;
   const int64_t t0 = (int64_t)blockIdx.x * INV_TILE;
@@ -511,14 +467,16 @@ __global__ void __launch_bounds__(512) inv_scatter_kernel(const Plan* __restrict
                                                           const uint32_t* __restrict__ Zp,
                                                           const Fields fl, int64_t n,
                                                           uint32_t* __restrict__ order) {
-  if (!plan->any) return;
+  if (!plan->any || plan->failed) return;
   extern __shared__ uint32_t slice[];  // [1 << FINE_SHIFT]
   const int64_t s0 = (int64_t)blockIdx.x << FINE_SHIFT;
   const int len = (int)((n - s0 < (1 << FINE_SHIFT)) ? n - s0 : (1 << FINE_SHIFT));
-  for (int i = threadIdx.x; i < len; i += blockDim.x)
+#pragma unroll 8
+  for (int i = threadIdx.x; i < len; i += 512)
     slice[__ldcs(Zv + s0 + i) & ((1u << FINE_SHIFT) - 1)] = __ldcs(Zp + s0 + i);
   __syncthreads();
-  for (int i = threadIdx.x; i < len; i += blockDim.x) {
+#pragma unroll 8
+  for (int i = threadIdx.x; i < len; i += 512) {
     const uint32_t v = (uint32_t)(s0 + i);
     order[s0 + i] = fl.n > 1 ? slice[i] - (uint32_t)__ldg(fl.off + field_of(fl, v)) : slice[i];
   }
@@ -533,8 +491,7 @@ __global__ void identity_kernel(const Plan* __restrict__ plan, uint32_t* order, 
 
 struct OrderWs {
   uint32_t *ka, *kb, *va, *vb;
-  unsigned int* th;
-  unsigned int* sums;
+  unsigned long long* look;  // per tile and digit (onesweep_kernel)
   unsigned int* ghist;
   unsigned int* cur;  // inverse permutation: coarse then fine slice cursors
   int64_t ncur;
@@ -546,13 +503,11 @@ OrderWs carve_order(void* base, int64_t n) {
   WsCarver c(base);
   OrderWs w;
   const int64_t ntiles = (n + SORT_TILE - 1) / SORT_TILE;
-  const int64_t m = ntiles * 256;
   w.ka = c.take<uint32_t>(n);
   w.kb = c.take<uint32_t>(n);
   w.va = c.take<uint32_t>(n);
   w.vb = c.take<uint32_t>(n);
-  w.th = c.take<unsigned int>(m);
-  w.sums = c.take<unsigned int>((m + SCAN_CHUNK - 1) / SCAN_CHUNK + 1);
+  w.look = c.take<unsigned long long>(ntiles * 256);
   w.ghist = c.take<unsigned int>(1024);
   w.ncur = ((int64_t)COARSE_BINS + (n >> FINE_SHIFT) + 1) * CUR_STRIDE;
   w.cur = c.take<unsigned int>(w.ncur);
@@ -579,11 +534,9 @@ int launch_order_fields(const float* f, int64_t n, const int64_t* foff, int nfie
   const Fields fl{foff, nfields};
   OrderWs w = carve_order(ws, n);
   const int64_t ntiles = (n + SORT_TILE - 1) / SORT_TILE;
-  const int64_t m = ntiles * 256;
-  const int64_t nsums = (m + SCAN_CHUNK - 1) / SCAN_CHUNK;
   static bool configured = false;
   if (!configured) {
-    if (cudaFuncSetAttribute(downsweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(onesweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(DownSmem)) != cudaSuccess ||
         cudaFuncSetAttribute(inv_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(uint32_t) << FINE_SHIFT)) != cudaSuccess)
@@ -597,16 +550,12 @@ int launch_order_fields(const float* f, int64_t n, const int64_t* foff, int nfie
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int64_t hb = std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
   hist_all_kernel<<<(unsigned)hb, 256, 0, s>>>(f, n, w.ghist, dstatus); count_launch();
-  plan_kernel<<<1, 32, 0, s>>>(w.ghist, n, nfields, w.plan); count_launch();
+  plan_kernel<<<1, 256, 0, s>>>(w.ghist, n, fl, w.plan); count_launch();
+  DMS_CUDA_OK(cudaMemsetAsync(w.look, 0, ntiles * 256 * sizeof(unsigned long long), s));
   const int passes = nfields > 256 ? 6 : (nfields > 1 ? 5 : 4);
   for (int p = 0; p < passes; ++p) {
-    upsweep_kernel<<<(unsigned)ntiles, SORT_NT, 0, s>>>(p, w.plan, f, w.ka, w.kb, w.va, w.vb, fl, n,
-                                                        ntiles, w.th); count_launch();
-    scan_reduce_kernel<<<(unsigned)nsums, SCAN_NT, 0, s>>>(p, w.plan, w.th, m, w.sums); count_launch();
-    scan_sums_kernel<<<1, SCAN_NT, 0, s>>>(p, w.plan, w.sums, nsums); count_launch();
-    scan_down_kernel<<<(unsigned)nsums, SCAN_NT, 0, s>>>(p, w.plan, w.th, m, w.sums); count_launch();
-    downsweep_kernel<<<(unsigned)ntiles, SORT_NT, sizeof(DownSmem), s>>>(
-        p, w.plan, f, w.ka, w.kb, w.va, w.vb, order, fl, n, ntiles, w.th, inverse); count_launch();
+    onesweep_kernel<<<(unsigned)ntiles, SORT_NT, sizeof(DownSmem), s>>>(
+        p, w.plan, f, w.ka, w.kb, w.va, w.vb, order, fl, n, w.look, inverse, dstatus); count_launch();
   }
   if (inverse) {
     // sorted payloads -> (vertex, position) by coarse slice (ka, kb) -> by
