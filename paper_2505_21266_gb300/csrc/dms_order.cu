@@ -482,11 +482,14 @@ __global__ void __launch_bounds__(512) inv_scatter_kernel(const Plan* __restrict
   }
 }
 
-__global__ void identity_kernel(const Plan* __restrict__ plan, uint32_t* order, int64_t n) {
-  if (plan->any) return;
+// no pass to run; also after a wait that ran out, so that what is launched
+// behind meets a permutation
+__global__ void identity_kernel(const Plan* __restrict__ plan, const Fields fl, uint32_t* order,
+                                int64_t n) {
+  if (plan->any && !plan->failed) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
-    order[i] = (uint32_t)i;
+    order[i] = (uint32_t)(fl.n > 1 ? i - __ldg(fl.off + field_of(fl, (uint32_t)i)) : i);
 }
 
 struct OrderWs {
@@ -572,7 +575,7 @@ int launch_order_fields(const float* f, int64_t n, const int64_t* foff, int nfie
                                                                            n, order); count_launch();
   }
   int64_t ib = std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
-  identity_kernel<<<(unsigned)ib, 256, 0, s>>>(w.plan, order, n); count_launch();
+  identity_kernel<<<(unsigned)ib, 256, 0, s>>>(w.plan, fl, order, n); count_launch();
   return launch_status();
 }
 
