@@ -1,12 +1,13 @@
 // Extremum-saddle persistence pairs D0 and D2 (Sec. 2.5, Alg. 1; Sec. 4.1-4.2).
 //
-// 1. v-path tracing, two walks per critical saddle, dealt to the lanes of a
-//    persistent grid as their previous walks end.  D0: from both vertices
-//    of a critical edge, follow desc[] (vertex -> paired edge -> other vertex)
-//    to a minimum.  D2: from both cofacets of a critical triangle follow the
-//    dual gradient (tet -> its paired facet -> that facet's other cofacet) to
-//    a critical tetrahedron, or to the virtual OUTSIDE node when the path
-//    leaves the grid.  Triplets whose two ends coincide are dropped.
+// 1. v-path tracing.  D0: from both vertices of a critical edge, follow desc[]
+//    (vertex -> paired edge -> other vertex) to a minimum.  D2: from both
+//    cofacets of a critical triangle follow the dual gradient (tet -> its
+//    paired facet -> that facet's other cofacet) to a critical tetrahedron, or
+//    to the virtual OUTSIDE node when the path leaves the grid.  The paths are
+//    first resolved by bricks of the grid in shared memory (every cell learns
+//    where its path leaves the brick, or its extremum), then each saddle hops
+//    from brick to brick.  Triplets whose two ends coincide are dropped.
 // 2. Pairing rounds.  Alg. 1 visits the saddles in increasing order and, with
 //    a union-find whose roots are the oldest extremum of each component,
 //    pairs the saddle with the younger root when it joins two components.
@@ -18,13 +19,14 @@
 //    every merge -- and therefore every pair -- is the one Alg. 1 makes;
 //    saddles whose ends already share a root are dropped, as in Alg. 1.
 //    The lightest live saddle overall qualifies, so each round makes progress.
-//    Per round: kernel 1 finds both roots (path halving) and records, per
+//    Per round: one phase finds both roots (path halving) and records, per
 //    root, the lightest saddle with one 64-bit atomicMax of
-//    (round << 44 | ~weight); kernel 2 merges the mutual ones and appends the
-//    rest to the next live list.
-// 3. Paired saddles are compacted in saddle-id order (block scans plus one
-//    device-wide scan) and written as dms_pair records; birth/death values
-//    are copied from the field.
+//    (round << 44 | ~weight); the other merges the mutual ones and appends the
+//    rest to the next live list.  A phase is a launch while very many saddles
+//    are live, the later rounds are one cooperative launch.
+// 3. Paired saddles are compacted in saddle-id order in one launch (a tile
+//    looks back at the counts of the tiles before it) and written as dms_pair
+//    records; birth/death values are copied from the field.
 //
 // Weights and ages are 44-bit integers ordered like the lexicographic keys
 // of Sec. 2.1: (order of the top vertex) followed by the ranks, among the
