@@ -42,6 +42,7 @@ constexpr int SORT_TILE = SORT_NT * SORT_ITEMS;  // 4096
 constexpr int SORT_WARPS = SORT_NT / 32;
 constexpr int kLookAhead = 4;           // tiles read at a time when looking back
 constexpr uint32_t kLookPolls = 1u << 22;
+constexpr unsigned int kNoTile = 0xFFFFFFFFu;  // in place of a ticket: nothing more is sorted
 
 enum : int { SRC_FIELD = 0, SRC_A = 1, SRC_B = 2, DST_A = 1, DST_B = 2, DST_ORDER = 3 };
 
@@ -222,7 +223,8 @@ static_assert(SORT_WARPS * 256 <= SORT_TILE, "the masks fit where the keys go");
 // count, 2 * pass + 2 when it is the count up to the tile's end.  Tickets are
 // drawn in order, so the tiles that a CTA waits for are running or done; the
 // waits are bounded all the same, and after one that ran out nothing more is
-// sorted.
+// sorted: other CTAs of the launch set `failed` while this one starts, so one
+// thread reads it, and the whole CTA leaves or stays by what that thread saw.
 // Bound by the shared-memory pipe (78 % of its peak: the masks, the counts,
 // the tile's staging) and by the latency of ranking, with DRAM at a third of
 // its rate.  The whole order took, at 1024^3, 512^3 quantised, 64^3 and 24^3,
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(SORT_NT, 4) onesweep_kernel(
     int pass, Plan* __restrict__ plan, const float* __restrict__ f, uint32_t* ka, uint32_t* kb,
     uint32_t* va, uint32_t* vb, uint32_t* __restrict__ order, const Fields fl, int64_t n,
     unsigned long long* look, bool inverse, int32_t* dstatus) {
-  if (!plan->active[pass] || plan->failed) return;
+  if (!plan->active[pass]) return;
   const int src = plan->src[pass], dst = plan->dst[pass];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   DownSmem& sm = *reinterpret_cast<DownSmem*>(smem_raw);
@@ -246,8 +248,10 @@ __global__ void __launch_bounds__(SORT_NT, 4) onesweep_kernel(
     (&sm.wh[0][0])[i] = 0;
     (&sm.peers[0][0])[i] = 0;
   }
-  if (threadIdx.x == 0) sm.tile = atomicAdd(&plan->ticket[pass], 1u);
+  if (threadIdx.x == 0)
+    sm.tile = *(volatile int*)&plan->failed ? kNoTile : atomicAdd(&plan->ticket[pass], 1u);
   __syncthreads();
+  if (sm.tile == kNoTile) return;
   const int64_t tile = sm.tile, tile0 = tile * SORT_TILE;
   const int64_t base = tile0 + (int64_t)warp * (32 * SORT_ITEMS);
   uint32_t key[SORT_ITEMS], val[SORT_ITEMS];
