@@ -35,6 +35,7 @@
 
 #include "dms_common.cuh"
 #include "dms_radix.cuh"
+#include "dms_rounds.cuh"
 #include "dms_scan.cuh"
 
 namespace dms {
@@ -929,26 +930,10 @@ __global__ void reset_nodes(Nodes nd, const int64_t* __restrict__ n_dev, int64_t
 // (117 M saddles) and 31.4 instead of 30.5 ms on 512^3 quantised noise; the
 // line lies where both ways cost the same (512 K to 10 M: within 1 %).
 constexpr int kRoundThreads = 512;
-constexpr unsigned int kSolo = 4096;           // live saddles that CTA 0 works alone
-constexpr int64_t kSoloNodes = 1 << 16;        // nodes that it sets back alone
 constexpr int64_t kOneLaunch = (int64_t)3 << 20;  // saddles up to which the rounds are one launch
 constexpr unsigned int kMaxExactRounds = 256;  // then the sorted finish, whatever is left
 constexpr unsigned int kMaxForestRounds = 64;  // components at least halve per round
 constexpr uint32_t kBarrierPolls = 1u << 23;
-
-// words of DiagWs::ctr
-enum : int {
-  kCtrLive = 0,      // saddles live after the walks
-  kCtrNext = 1,      // live saddles of the rounds of one launch per phase: with kCtrLive in turn
-  kCtrForest = 2,    // saddles of the spanning forest
-  kCtrChanged = 3,   // (self-correcting pairing)
-  kCtrBig = 4,       // saddles left to the device-wide sorted finish (batch)
-  kCtrRound = 8,     // three live counts in turn
-  kCtrLeft = 11,     // saddles left live by the exact rounds
-  kCtrBarrier = 12,
-  kCtrAbort = 13,
-  kCtrWords = 16
-};
 
 struct Rounds {
   Tri T;
@@ -1041,8 +1026,7 @@ __global__ void __launch_bounds__(kRoundThreads, 4) pair_rounds(const Rounds R, 
   uint32_t *cur = R.cur, *nxt = R.nxt;
   bool solo = gridDim.x == 1, forest = R.forest != nullptr, found = R.first_found;
   for (;;) {
-    // (many nodes are set back by the whole grid)
-    if (!solo && n <= kSolo && (!forest || nn <= kSoloNodes)) {
+    if (!solo && goes_solo(n, nn, forest)) {
       if (blockIdx.x != 0) return;
       solo = true;
     }
@@ -1057,7 +1041,7 @@ __global__ void __launch_bounds__(kRoundThreads, 4) pair_rounds(const Rounds R, 
         nd.best[i] = 0ull;
       }
       n = __ldcg(ctr + kCtrForest);
-      if (first < 3) ctr[kCtrRound + first] = 0;
+      if (first < 3) ctr[count_word(first, solo)] = 0;
       nxt = R.cur;
       cur = R.forest;
       round = 1;
@@ -1070,9 +1054,9 @@ __global__ void __launch_bounds__(kRoundThreads, 4) pair_rounds(const Rounds R, 
       if (!round_sync(ctr, epoch, solo)) break;
     }
     found = false;
-    // round r counts in word r % 3; word (r + 1) % 3 was last read two rounds ago
-    unsigned int* const nxt_n = ctr + kCtrRound + round % 3;
-    if (first == 0) ctr[kCtrRound + (round + 1) % 3] = 0;
+    // the next round's word was last read two rounds ago
+    unsigned int* const nxt_n = ctr + count_word(round, solo);
+    if (first == 0) ctr[count_word(round + 1, solo)] = 0;
     // CTA-uniform passes: every thread reaches the appends
     for (unsigned int base = first - threadIdx.x; base < n; base += step) {
       const unsigned int j = base + threadIdx.x;
