@@ -31,6 +31,8 @@
 // Weights and ages are 44-bit integers ordered like the lexicographic keys
 // of Sec. 2.1: (order of the top vertex) followed by the ranks, among the
 // lower neighbours of that top vertex, of the other vertices.
+#include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "dms_common.cuh"
@@ -1088,16 +1090,21 @@ __global__ void __launch_bounds__(kRoundThreads, 4) pair_rounds(const Rounds R, 
 // launches pair_rounds for at most n live saddles (its own words of ctr are
 // zero: all from kCtrRound on)
 int launch_rounds(const Rounds& R, int64_t n, int32_t* dstatus, cudaStream_t s) {
-  static int blocks = 0;
+  // the device's resident CTAs: asked once per device, by any thread (they find the same)
+  constexpr int kDevices = 64;
+  static std::atomic<int> resident[kDevices];
+  int dev = 0, blocks = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return DMS_ERR_CUDA;
+  if (dev < kDevices) blocks = resident[dev].load(std::memory_order_relaxed);
   if (blocks == 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+    int sms = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_rounds, kRoundThreads, 0) !=
             cudaSuccess ||
         per_sm < 1)
       return DMS_ERR_CUDA;
     blocks = sms * per_sm;
+    if (dev < kDevices) resident[dev].store(blocks, std::memory_order_relaxed);
   }
   const unsigned grid =
       n <= (int64_t)kSolo ? 1u

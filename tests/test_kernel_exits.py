@@ -1,4 +1,4 @@
-"""Early exits of the CTA-wide kernels, read off their source: a word that
+"""Launches and early exits, read off their source.  A word that
 other CTAs of the same launch may write is no ground for a thread to leave
 ahead of a barrier by itself, since the threads of one CTA may see different
 values.  (What such a kernel does after a disagreement is an access out of
@@ -33,3 +33,16 @@ def test_sort_pass_leaves_as_a_whole():
     assert rest.index("if (sm.tile == kNoTile) return") < rest.index("tile = sm.tile")
     # further on it is only ever set
     assert set(re.findall(r"failed[^;]*", rest)) == {"failed = 1"}
+
+
+def test_cooperative_grid_is_kept_per_device():
+    """launch_rounds: what it keeps between calls (how many of its CTAs a
+    device holds at once) is kept by device and may be read and written by
+    several threads; a grid that is too large for the current device is
+    refused at its launch, one from a race is anything."""
+    s = open(os.path.join(CSRC, "dms_pairs.cu")).read()
+    at = s.index("int launch_rounds(")
+    body = s[at:s.index("\n}\n", at)]
+    kept = re.findall(r"static (?!constexpr|const )[^;]*;", body)
+    assert all(re.match(r"static std::atomic<int> \w+\[kDevices\];", k) for k in kept), kept
+    assert body.index("cudaGetDevice(&dev)") < body.index("resident[dev]")
