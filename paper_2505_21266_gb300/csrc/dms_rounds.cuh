@@ -13,8 +13,7 @@
 
 namespace dms {
 
-constexpr unsigned int kSolo = 4096;     // live saddles that CTA 0 works alone
-constexpr int64_t kSoloNodes = 1 << 16;  // nodes that it sets back alone
+constexpr unsigned int kSolo = 4096;  // live saddles that CTA 0 works alone
 
 // words of DiagWs::ctr
 enum : int {
@@ -38,9 +37,13 @@ DMS_ROUNDS_HD int count_word(unsigned int round, bool solo) {
   return (solo ? kCtrSolo : kCtrRound) + (int)(round % 3);
 }
 
-// whether CTA 0 goes on alone with n live saddles of nn nodes
+// whether CTA 0 goes on alone with n live saddles of nn nodes.  From the forest's
+// rounds it goes on to the exact rounds on the forest's saddles, up to nn - 1:
+// those have to be few as well, however few are live before.  With the line at
+// 65,536 nodes instead, the D0/D2 stage of noise took 1.00 ms at 64^3 and 2.50
+// at 96^3 (17 K and 58 K nodes); it takes 0.66 and 0.90.
 DMS_ROUNDS_HD bool goes_solo(unsigned int n, int64_t nn, bool forest) {
-  return n <= kSolo && (!forest || nn <= kSoloNodes);  // (many nodes are set back by the whole grid)
+  return n <= kSolo && (!forest || nn <= (int64_t)kSolo + 1);
 }
 
 }  // namespace dms

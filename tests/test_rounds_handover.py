@@ -37,8 +37,8 @@ class Sim:
     round, then 0; exact: the forest's saddles, then those left after each
     exact round, then 0."""
 
-    def __init__(self, lib, count_word, nn, forest, exact):
-        self.lib, self.count_word, self.nn = lib, count_word, nn
+    def __init__(self, lib, count_word, goes_solo, nn, forest, exact):
+        self.lib, self.count_word, self.goes_solo, self.nn = lib, count_word, goes_solo, nn
         self.plan = {"forest": forest, "exact": exact}
         self.ctr = [0] * lib.host_words()
         self.ctr[lib.host_forest_word()] = exact[0]
@@ -50,7 +50,7 @@ class Sim:
         ctr, solo, forest, rnd, epoch = self.ctr, False, True, 1, 0
         n, at = self.plan["forest"][0], 0
         while True:
-            if not solo and self.lib.host_goes_solo(n, self.nn, forest):
+            if not solo and self.goes_solo(n, self.nn, forest):
                 if b != 0:
                     return
                 solo = True
@@ -140,10 +140,10 @@ def _orders():
         yield lambda ready: 0 if 0 in ready and rng.random() < ahead else rng.choice(ready)
 
 
-def _ok(lib, count_word):
+def _ok(lib, count_word, goes_solo):
     for nn, forest, exact in PLANS:
         for order in _orders():
-            s = Sim(lib, count_word, nn, forest, exact)
+            s = Sim(lib, count_word, goes_solo, nn, forest, exact)
             if not s.run(order):
                 return False
             alone = [i for i, w in enumerate(s.worked) if w[1]]
@@ -156,12 +156,29 @@ def _ok(lib, count_word):
     return True
 
 
+def _many_after_few(n, nn, forest):
+    """A hand-over that lets CTA 0 meet up to 65,536 saddles alone."""
+    return n <= 4096 and (not forest or nn <= 65_536)
+
+
 def test_late_readers_leave(lib):
-    assert _ok(lib, lambda r, solo: lib.host_count_word(r, int(solo)))
+    for goes_solo in (lib.host_goes_solo, _many_after_few):
+        assert _ok(lib, lambda r, solo: lib.host_count_word(r, int(solo)), goes_solo)
 
 
 def test_shared_words_are_caught(lib):
-    assert not _ok(lib, lambda r, solo: lib.host_first_round_word() + r % 3)
+    assert not _ok(lib, lambda r, solo: lib.host_first_round_word() + r % 3, _many_after_few)
+
+
+def test_few_saddles_alone(lib):
+    """CTA 0 alone never meets more than kSolo saddles: neither those live at
+    the hand-over, nor, from the forest's rounds, the forest's (nodes - 1)."""
+    few = lib.host_solo()
+    for nn in (2, few, few + 1, few + 2, 2 * few, 60_000, 65_536, 65_537, 1 << 20):
+        for n in (1, few - 1, few, few + 1, 1 << 20):
+            for forest in (False, True):
+                alone = lib.host_goes_solo(n, nn, int(forest))
+                assert bool(alone) == (n <= few and (not forest or nn - 1 <= few)), (n, nn, forest)
 
 
 def test_words_do_not_overlap(lib):
