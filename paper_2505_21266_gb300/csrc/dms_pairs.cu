@@ -35,6 +35,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "dms_bricks.cuh"
 #include "dms_common.cuh"
 #include "dms_radix.cuh"
 #include "dms_rounds.cuh"
@@ -137,60 +138,6 @@ __device__ __forceinline__ int tet_type(int c1, int c2) {
   return (c1 >> 1) * 2 + ((c2 ^ c1) > (7 ^ c2) ? 1 : 0);
 }
 
-// One step of an ascending dual path, tabulated.  Tet type k (chain
-// 0 < c1 < c2 < 7 of its anchor cube) paired with the facet that omits
-// chain vertex code - 1 leaves through that facet into the other tet on it:
-//  * code 1 omits the anchor: the next tet is anchored at anchor + c1, chain
-//    (c2 ^ c1, 7 ^ c1);
-//  * code 4 omits the top: anchored at anchor - (7 ^ c2), chain
-//    (7 ^ c2, (7 ^ c2) | c1);
-//  * code 2 / 3 omit c1 / c2: same anchor, chain (c2 ^ c1, c2) / (c1, c1 | (7 ^ c2)).
-// entry(4k + code - 1): next type (bits 0-2), anchor step corner (3-5), step
-// sign (6-7: 0 none, 1 plus, 2 minus).
-namespace dual_step_detail {
-constexpr int c1_of(int k) { return (0x442211 >> (4 * k)) & 15; }
-constexpr int c2_of(int k) { return (0x656353 >> (4 * k)) & 15; }
-constexpr int type_of(int c1, int c2) { return (c1 >> 1) * 2 + ((c2 ^ c1) > (7 ^ c2) ? 1 : 0); }
-constexpr uint64_t entry(int e) {
-  const int k = e / 4, code = e % 4 + 1, c1 = c1_of(k), c2 = c2_of(k);
-  int stp = 0, sg = 0, n1 = 0, n2 = 0;
-  if (code == 1) { stp = c1; sg = 1; n1 = c2 ^ c1; n2 = 7 ^ c1; }
-  else if (code == 4) { stp = 7 ^ c2; sg = 2; n1 = stp; n2 = stp | c1; }
-  else if (code == 2) { n1 = c2 ^ c1; n2 = c2; }
-  else { n1 = c1; n2 = c1 | (7 ^ c2); }
-  return (uint64_t)(type_of(n1, n2) | (stp << 3) | (sg << 6));
-}
-}  // namespace dual_step_detail
-// ---------------------------------------------------------------------------
-// v-paths by bricks.
-//
-// A path (vertex -> paired edge -> other vertex; tet -> paired facet -> other
-// cofacet) is followed cell by cell only inside bricks of up to 8192 cells, in
-// shared memory, for all cells of a brick at once: every cell then knows where
-// its path ends or leaves the brick, and a walk hops from brick to brick.
-// Every cell has one word:
-//   bit 31 set    the end: bits 0..30 the node (0 for OUTSIDE in the dual)
-//   bit 31 clear  where the path goes on: bits 13..18 the brick (two bits per
-//                 axis: 0, 1, 2 for the one before, this one, the next), bits
-//                 0..12 the cell in it
-// mark_ends gives the cells at path ends (minima, critical tets) their nodes
-// first; resolve_paths reads them there.
-// Followed cell by cell through memory, one load and one claim by
-// compare-and-swap per step, a walk was a chain of 3 (vertices) and 10 (tets)
-// dependent steps on average on noise, up to 400 on smooth fields, 1 us each;
-// hops are 1.3 to 2.7 on average, up to 27.  Resolving all cells costs about
-// 100 instructions per tet and a word per cell written, which noise, whose
-// paths are short, pays back in fewer random reads: D0/D2 stage 64^3 mixture
-// 705 -> 356 us, 128^3 smooth 953 -> 368 us, 16384^2 37.8 -> 30.8 ms, 512^3
-// ties 28.9 -> 25.1 ms, 1024^3 87.7 -> 75.8 ms (of it a dual step as a sum on
-// the cell's word, in place of packed coordinates: 1.5).  Following every cell to its
-// end in turn instead of doubling took 147 ms there.
-// ---------------------------------------------------------------------------
-constexpr uint32_t kEnd = 0x80000000u;
-constexpr uint32_t kNoMark = kEnd | 0x7FFFFFFFu;  // an end without a node, or bad data
-constexpr uint32_t kLoop = kEnd | 0x7FFFFFFEu;    // a path that does not end (bad data)
-constexpr uint32_t kFinal = 0x40000000u;          // (in shared memory) a way on, out of the brick
-
 __global__ void mark_ends(const int64_t* __restrict__ list, const int64_t* n_dev, int64_t n_host,
                           uint32_t node0, uint32_t* path) {
   const int64_t n = n_dev ? *n_dev : n_host;
@@ -261,26 +208,6 @@ __device__ __forceinline__ void tri_cofacets(const Grid& g, int64_t a, int k, in
   }
 }
 
-// one field for the whole call
-struct OneField {
-  Grid g;
-  __device__ __forceinline__ void get(int64_t, Grid& out, int64_t& off) const {
-    out = g;
-    off = 0;
-  }
-  // brick id of 2^lx x 2^ly x 2^lz vertices: its field, its place in it
-  __device__ __forceinline__ void brick(int64_t id, int lx, int ly, int lz, Grid& out, int64_t& off,
-                                        int& bx, int& by, int& bz) const {
-    get(0, out, off);
-    const uint32_t tx = (uint32_t)((g.nx + (1 << lx) - 1) >> lx), ty = (uint32_t)((g.ny + (1 << ly) - 1) >> ly);
-    const uint32_t i = (uint32_t)id, r = i / tx;
-    bx = (int)(i - r * tx);
-    bz = (int)(r / ty);
-    by = (int)(r - (uint32_t)bz * ty);
-    (void)lz;
-  }
-};
-
 // a batch: the field that holds an anchor or a brick, by binary search
 struct ManyFields {
   const dms_field_desc* fd;
@@ -322,132 +249,6 @@ __device__ __forceinline__ int64_t slot_delta_g(const Grid& g, int s) {
   const int64_t d = (c & 1) + ((c >> 1) & 1) * g.nx + ((c >> 2) & 1) * g.sxy;
   return s < 7 ? d : -d;
 }
-
-// A cell of a brick: its vertex's coordinates in one word, eight bits per
-// axis, each offset by the brick's extent, so that after a step the bits above
-// the coordinate's say which brick it is in: 0, 1 (this one) or 2.
-template <class P>
-__device__ __forceinline__ uint32_t packed_coords(int lv) {
-  return ((lv & ((1 << P::LX) - 1)) + (1 << P::LX)) |
-         (((lv >> P::LX) & ((1 << P::LY) - 1)) + (1 << P::LY)) << 8 |
-         ((lv >> (P::LX + P::LY)) + (1 << P::LZ)) << 16;
-}
-__device__ __forceinline__ constexpr uint32_t packed_step(int dx, int dy, int dz) {
-  return (uint32_t)(dx + dy * 256 + dz * 65536);
-}
-// cell k of the vertex at c as a word: a cell of the brick, or a way out of it
-template <class P>
-__device__ __forceinline__ uint32_t brick_word(uint32_t c, int k) {
-  const uint32_t lv = (c & ((1u << P::LX) - 1)) | (c >> 8 & ((1u << P::LY) - 1)) << P::LX |
-                      (c >> 16 & ((1u << P::LZ) - 1)) << (P::LX + P::LY);
-  const uint32_t dir = (c >> P::LX & 3u) | (c >> (8 + P::LY) & 3u) << 2 | (c >> (16 + P::LZ) & 3u) << 4;
-  const uint32_t local = lv * P::K + k;
-  return dir == 21u ? local : kFinal | dir << 13 | local;
-}
-// is the vertex at c inside [0, mx) x [0, my) x [0, mz) of the brick at (x0, y0, z0)
-template <class P>
-__device__ __forceinline__ bool inside(uint32_t c, int x0, int y0, int z0, uint32_t mx, uint32_t my,
-                                       uint32_t mz) {
-  return (uint32_t)(x0 + (int)(c & 255u) - (1 << P::LX)) < mx &&
-         (uint32_t)(y0 + (int)(c >> 8 & 255u) - (1 << P::LY)) < my &&
-         (uint32_t)(z0 + (int)(c >> 16) - (1 << P::LZ)) < mz;
-}
-// (A policy's cells() replaces the words that are not kNoMark.)
-// the word of the end of a path: the node that mark_ends gave the cell (ends
-// that are not in the list have none: bad data)
-__device__ __forceinline__ uint32_t end_word(const uint32_t* path, int64_t cell, const int64_t* list,
-                                             int64_t n, uint32_t node0) {
-  const uint32_t w = path[cell];
-  const int64_t i = (int64_t)(w & ~kEnd) - node0;
-  return (w & kEnd) && i >= 0 && i < n && __ldg(list + i) == cell ? w : kNoMark;
-}
-
-// D0: descending paths from vertex to vertex, to a minimum
-template <class F>
-struct DescPaths {
-  static constexpr int K = 1, LX = 4, LY = 4, LZ = 4;
-  F fields;
-  const uint8_t* desc;
-  const int64_t* ends;  // the path ends' cells, their number (n_dev or n)
-  const int64_t* n_dev;
-  int64_t n;
-  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
-                                        int y0, int z0, bool border, uint32_t (&w)[K]) const {
-    const int d = __ldg(desc + v);
-    if (d >= 14) {
-      if (d == 15) w[0] = end_word(path, v, ends, n_dev ? *n_dev : n, 0);
-      return;
-    }
-    const int c = (0x7653421 >> (4 * (d < 7 ? d : d - 7))) & 15, s = d < 7 ? 1 : -1;
-    const uint32_t to = packed_coords<DescPaths>(lv) +
-                        s * packed_step(c & 1, (c >> 1) & 1, (c >> 2) & 1);
-    const bool out = border && !inside<DescPaths>(to, x0, y0, z0, (uint32_t)g.nx, (uint32_t)g.ny, (uint32_t)g.nz);
-    if (!out) w[0] = brick_word<DescPaths>(to, 0);  // (outside: bad data)
-  }
-};
-
-// the steps of the dual paths from tet type k with code c, at 4 k + c - 1, and
-// the type they lead to (codes 2 and 3 stay at the anchor)
-struct DualSteps {
-  uint32_t step[24];
-  uint8_t type[24];
-};
-constexpr DualSteps make_dual_steps() {
-  DualSteps t{};
-  for (int e = 0; e < 24; ++e) {
-    const uint64_t w = dual_step_detail::entry(e);
-    const int c = (int)(w >> 3) & 7, sg = (int)(w >> 6) == 1 ? 1 : ((int)(w >> 6) == 2 ? -1 : 0);
-    t.step[e] = (uint32_t)(sg * ((c & 1) + ((c >> 1) & 1) * 256 + ((c >> 2) & 1) * 65536));
-    t.type[e] = (uint8_t)(w & 7);
-  }
-  return t;
-}
-
-// D2: ascending dual paths from tet to tet, to a critical one or out of the
-// grid (node 0, OUTSIDE)
-template <class F>
-struct DualPaths {
-  static constexpr int K = 6, LX = 4, LY = 3, LZ = 3;
-  F fields;
-  const uint64_t* rec;
-  const int64_t* ends;
-  const int64_t* n_dev;
-  int64_t n;
-  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
-                                        int y0, int z0, bool border, uint32_t (&w)[K]) const {
-    constexpr DualSteps st = make_dual_steps();
-    constexpr int L[3] = {LX, LY, LZ};
-    const uint32_t hi = (uint32_t)(__ldg(rec + v) >> 32), at = packed_coords<DualPaths>(lv);
-    // a step goes up or down one axis: what it adds to the cell's word, with
-    // the wrap and the brick where it leaves this one
-    uint32_t up[3], down[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int shift = a == 0 ? 0 : (a == 1 ? LX : LX + LY), last = (1 << L[a]) - 1;
-      const int at_axis = (lv >> shift) & last, one = K << shift;
-      up[a] = at_axis == last ? kFinal + ((21 + (1 << 2 * a)) << 13) - last * one : one;
-      down[a] = at_axis == 0 ? kFinal + ((21 - (1 << 2 * a)) << 13) + last * one : 0u - one;
-    }
-    const uint32_t base = (uint32_t)lv * K;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const uint32_t code = (hi >> (1 + 3 * k)) & 7u;
-      if (code == 7u) {
-        w[k] = end_word(path, v * 6 + k, ends, n_dev ? *n_dev : n, 1);
-      } else if (code >= 1u && code <= 4u) {  // (else no tet there, or bad data)
-        const int u = dual_step_detail::c1_of(k) >> 1, d = (7 ^ dual_step_detail::c2_of(k)) >> 1;
-        const uint32_t add = code == 1u ? up[u] + st.type[4 * k]
-                             : (code == 2u ? st.type[4 * k + 1]
-                                : (code == 3u ? st.type[4 * k + 2] : down[d] + st.type[4 * k + 3]));
-        // (tet anchors lie below the last vertex in every axis)
-        const bool out = border && !inside<DualPaths>(
-                                       at + (code == 1u ? st.step[4 * k] : (code == 4u ? st.step[4 * k + 3] : 0u)),
-                                       x0, y0, z0, (uint32_t)(g.nx - 1), (uint32_t)(g.ny - 1), (uint32_t)(g.nz - 1));
-        w[k] = out ? kEnd : base + add;  // out: OUTSIDE
-      }
-    }
-  }
-};
 
 // One CTA per brick: the words of all its cells, by pointer doubling.  A word
 // is always a cell further along the path, so no barrier is needed between
@@ -523,53 +324,11 @@ __global__ void __launch_bounds__(kBrickThreads) resolve_paths(const P p, uint32
   }
 }
 
-template <class P>
-int64_t brick_count(int64_t nx, int64_t ny, int64_t nz) {
-  return ((nx + (1 << P::LX) - 1) >> P::LX) * ((ny + (1 << P::LY) - 1) >> P::LY) *
-         ((nz + (1 << P::LZ) - 1) >> P::LZ);
-}
-
-// a walk: the word of its cell and the brick of that cell
-struct Walk {
-  uint32_t w;
-  int bx, by, bz;
-};
-template <class P>
-__device__ __forceinline__ Walk walk_from(const uint32_t* path, const Grid& g, int64_t v, int x, int y, int z,
-                                          int k) {
-  return Walk{__ldg(path + v * P::K + k), x >> P::LX, y >> P::LY, z >> P::LZ};
-}
-template <class P>
-__device__ __forceinline__ void walk_hop(const uint32_t* path, const Grid& g, int64_t off, Walk& a) {
-  const uint32_t local = a.w & 8191u, lv = local / P::K;
-  a.bx += (int)(a.w >> 13 & 3u) - 1;
-  a.by += (int)(a.w >> 15 & 3u) - 1;
-  a.bz += (int)(a.w >> 17 & 3u) - 1;
-  const int x = (a.bx << P::LX) + (int)(lv & ((1 << P::LX) - 1));
-  const int y = (a.by << P::LY) + (int)((lv >> P::LX) & ((1 << P::LY) - 1));
-  const int z = (a.bz << P::LZ) + (int)(lv >> (P::LX + P::LY));
-  a.w = __ldg(path + (off + x + g.nx * y + g.sxy * z) * P::K + (local - lv * P::K));
-}
 __device__ __forceinline__ uint32_t walk_end(const Walk& a, int32_t* dstatus) {
   if (a.w < kLoop) return a.w & ~kEnd;
   set_status(dstatus, a.w == kLoop ? DMS_ERR_TIMEOUT : DMS_ERR_ARG);  // bad data
   return 0;
 }
-// both walks of a saddle to their ends, their loads in flight together (a
-// path through more bricks than there are cells loops: bad data)
-template <class P>
-__device__ __forceinline__ void walk_both(const uint32_t* path, const Grid& g, int64_t off, Walk& a, Walk& b) {
-  int64_t left = g.n * P::K;
-  while (!(a.w & kEnd) || !(b.w & kEnd)) {
-    if (!(a.w & kEnd)) walk_hop<P>(path, g, off, a);
-    if (!(b.w & kEnd)) walk_hop<P>(path, g, off, b);
-    if (--left < 0) {
-      a.w = a.w & kEnd ? a.w : kLoop;
-      b.w = b.w & kEnd ? b.w : kLoop;
-    }
-  }
-}
-
 // the saddle's record with its weight and ends, live where they differ.  With
 // tag set it also does the first round's search of the pairing rounds (every
 // node is still its own root): both ends are the roots and are tagged with the
@@ -2167,7 +1926,6 @@ struct Grid2d {
   int64_t nx, ny, n;
 };
 
-__device__ __forceinline__ int corner2(int s) { return (s % 3) + 1; }  // {1,2,3}
 __device__ __forceinline__ int64_t cdelta2(const Grid2d& g, int c) {
   return (c & 1) + ((c >> 1) & 1) * g.nx;
 }
@@ -2231,56 +1989,6 @@ __global__ void init_nodes_d1_2d(Grid2d g, const uint32_t* __restrict__ order,
   const uint64_t key = ((uint64_t)o[it] << 8) | (h << 4) | l;
   nd.age[i] = (kMask44 - key) + 1;
 }
-
-// D0: down the vertex-edge pairs (desc) to a minimum
-struct DescPaths2d {
-  static constexpr int K = 1, LX = 5, LY = 5, LZ = 0;
-  OneField fields;
-  const uint8_t* desc;
-  const int64_t* ends;
-  int64_t n;
-  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
-                                        int y0, int, bool, uint32_t (&w)[K]) const {
-    const int d = __ldg(desc + v);
-    if (d >= 6) {
-      if (d == 15) w[0] = end_word(path, v, ends, n, 0);
-      return;
-    }
-    const int c = corner2(d), s = d < 3 ? 1 : -1;
-    const uint32_t to = packed_coords<DescPaths2d>(lv) + s * packed_step(c & 1, (c >> 1) & 1, 0);
-    const bool in = inside<DescPaths2d>(to, x0, y0, 0, (uint32_t)g.nx, (uint32_t)g.ny, 1u);
-    if (in) w[0] = brick_word<DescPaths2d>(to, 0);  // (outside: bad data)
-  }
-};
-
-// D1: from a triangle through the edge it is paired with to that edge's other
-// triangle, up to a maximum (node j + 1) or out of the grid (OUTSIDE, node 0)
-struct DualPaths2d {
-  static constexpr int K = 2, LX = 5, LY = 5, LZ = 0;
-  OneField fields;
-  const uint16_t* rec;
-  const int64_t* ends;
-  int64_t n;
-  __device__ __forceinline__ void cells(const Grid& g, const uint32_t* path, int64_t v, int lv, int x0,
-                                        int y0, int, bool, uint32_t (&w)[K]) const {
-    const uint32_t rw = __ldg(rec + v), at = packed_coords<DualPaths2d>(lv);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const uint32_t code = (rw >> (9 + 3 * k)) & 7u;
-      if (code == 7u) {
-        w[k] = end_word(path, v * 2 + k, ends, n, 1);
-      } else if (code >= 1u && code <= 3u) {  // (else no triangle there, or bad data)
-        // across the facet that omits chain vertex code - 1: the diagonal
-        // (code 2): the square's other triangle; type 0 (code 1 / 3): the
-        // square to the right / below; type 1: above / to the left
-        const uint32_t to = at + (code == 2u ? 0u : (code == 1u ? (k == 0 ? packed_step(1, 0, 0) : packed_step(0, 1, 0))
-                                                          : (k == 0 ? packed_step(0, -1, 0) : packed_step(-1, 0, 0))));
-        const bool in = inside<DualPaths2d>(to, x0, y0, 0, (uint32_t)(g.nx - 1), (uint32_t)(g.ny - 1), 1u);
-        w[k] = in ? brick_word<DualPaths2d>(to, 1 - k) : kEnd;
-      }
-    }
-  }
-};
 
 __host__ __device__ __forceinline__ Grid grid_of2d(const Grid2d& g) { return Grid{g.nx, g.ny, 1, g.n, g.n}; }
 
