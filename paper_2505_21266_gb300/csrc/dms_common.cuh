@@ -6,11 +6,15 @@
 #include <cuda_runtime.h>
 
 #include "../../include/dms.h"
-#include "dms_grid.cuh"
 
 namespace dms {
 
 constexpr int kSlots = 14;  // neighbours of a vertex in the Freudenthal triangulation
+
+struct Grid {
+  int64_t nx, ny, nz, n;
+  int64_t sxy;  // nx*ny
+};
 
 inline bool make_grid(dms_dims d, Grid* g) {
   if (d.nx < 2 || d.ny < 2 || d.nz < 2) return false;
