@@ -129,6 +129,16 @@ DMS_HD uint32_t end_word(const uint32_t* path, int64_t cell, const int64_t* list
   return (w & kEnd) && i >= 0 && i < n && ro(list + i) == cell ? w : kNoMark;
 }
 
+// a cell that a path is followed to without words: its vertex, its number there,
+// and 0 or, at the path's end, the end's word
+struct Cell {
+  uint32_t w;
+  int x, y, z, k;
+};
+DMS_HD bool within(const Cell& c, int64_t mx, int64_t my, int64_t mz) {
+  return (uint32_t)c.x < (uint32_t)mx && (uint32_t)c.y < (uint32_t)my && (uint32_t)c.z < (uint32_t)mz;
+}
+
 // D0: descending paths from vertex to vertex, to a minimum
 template <class F>
 struct DescPaths {
@@ -150,6 +160,20 @@ struct DescPaths {
                         s * packed_step(c & 1, (c >> 1) & 1, (c >> 2) & 1);
     const bool out = border && !inside<DescPaths>(to, x0, y0, z0, (uint32_t)g.nx, (uint32_t)g.ny, (uint32_t)g.nz);
     if (!out) w[0] = brick_word<DescPaths>(to, 0);  // (outside: bad data)
+  }
+  // the same for one cell
+  DMS_HD void step(const Grid& g, const uint32_t* path, int64_t v, Cell& c) const {
+    const int d = ro(desc + v);
+    c.w = kNoMark;
+    if (d >= 14) {
+      if (d == 15) c.w = end_word(path, v, ends, n_dev ? *n_dev : n, 0);
+      return;
+    }
+    const int o = (0x7653421 >> (4 * (d < 7 ? d : d - 7))) & 15, s = d < 7 ? 1 : -1;
+    c.x += s * (o & 1);
+    c.y += s * ((o >> 1) & 1);
+    c.z += s * ((o >> 2) & 1);
+    if (within(c, g.nx, g.ny, g.nz)) c.w = 0;  // (outside: bad data)
   }
 };
 
@@ -213,6 +237,21 @@ struct DualPaths {
         w[k] = out ? kEnd : base + add;  // out: OUTSIDE
       }
     }
+  }
+  DMS_HD void step(const Grid& g, const uint32_t* path, int64_t v, Cell& c) const {
+    const uint32_t code = (uint32_t)(ro(rec + v) >> (33 + 3 * c.k)) & 7u;
+    c.w = kNoMark;
+    if (code == 7u) c.w = end_word(path, v * 6 + c.k, ends, n_dev ? *n_dev : n, 1);
+    if (code < 1u || code > 4u) return;
+    const int c1 = dual_step_detail::c1_of(c.k), c2 = dual_step_detail::c2_of(c.k);
+    const int o = code == 1u ? c1 : (code == 4u ? 7 ^ c2 : 0), s = code == 1u ? 1 : -1;
+    const int n1 = code == 3u ? c1 : (code == 4u ? 7 ^ c2 : c2 ^ c1);
+    const int n2 = code == 1u ? 7 ^ c1 : (code == 2u ? c2 : c1 | (7 ^ c2));
+    c.k = dual_step_detail::type_of(n1, n2);
+    c.x += s * (o & 1);
+    c.y += s * ((o >> 1) & 1);
+    c.z += s * ((o >> 2) & 1);
+    c.w = within(c, g.nx - 1, g.ny - 1, g.nz - 1) ? 0 : kEnd;  // out: OUTSIDE
   }
 };
 
@@ -323,6 +362,62 @@ DMS_HD void walk_both(Path path, const Grid& g, int64_t off, Walk& a, Walk& b) {
   }
   if (!(a.w & kEnd)) a.w = walk_on<P>(path, g, off, a);
   if (!(b.w & kEnd)) b.w = walk_on<P>(path, g, off, b);
+}
+
+// ---------------------------------------------------------------------------
+// Few saddles on a large grid: paths cell by cell, no brick resolved.
+//
+// Walks that meet go on as one.  One vertex in eight is a landmark: the first
+// walk at a cell of it claims the cell's word, a later one stops there with a
+// link to the first.  So only the landmarks' words need clearing, and a walk
+// goes only a few steps along a path that another has taken.  Words: kNoMark
+// free, kEnd | node an end (mark_ends), kLink | walk claimed.  A walk's result:
+// an end, a link, or 0: a path, or a chain of links, too long for this (a walk
+// that loops, of bad data, among them), whose saddle waits for the bricks.
+//
+// Both bounds keep winding paths, one dependent load of 0.7 us per cell, from
+// costing more than a few ms ahead of the bricks; smooth fields of 1024^3
+// stay below.  Landmarks are 8 in a row of every 64, so that clearing writes
+// whole sectors: D0/D2 stage of 1024^3 mixtures with noise 0, 1e-3 and 2e-3
+// (2e-7, 2.3e-3 and 9e-3 saddles per vertex) 3.7, 7.3 and 17.8 ms; one in 16
+// anywhere 7.9, 12.2 and 24.6; 4 of 64 3.3, 7.4 and 19.4; 16 of 64 4.7, 8.4
+// and 18.6; without claims 1.5, 16.0 and 58.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kLink = 0x40000000u;  // (with fewer than 2^30 walks)
+constexpr int kFewSteps = 4096, kFewLinks = 4096;
+constexpr int kRun = 64, kGroup = 8;
+DMS_HD uint32_t landmarks_of(int64_t run) {  // place of a run's first landmark, by a hash
+  return ((uint32_t)run * 2654435761u) / (uint32_t)(0x100000000ull * kGroup / kRun) * kGroup;
+}
+DMS_HD bool is_landmark(int64_t v) { return ((uint32_t)v % kRun) / kGroup * kGroup == landmarks_of(v / kRun); }
+DMS_HD uint32_t claim(uint32_t* word, uint32_t me) {  // the word as it was
+#ifdef __CUDA_ARCH__
+  return atomicCAS(word, kNoMark, me);
+#else
+  const uint32_t w = *word;
+  if (w == kNoMark) *word = me;
+  return w;
+#endif
+}
+// walk number j from cell c: its result
+template <class P>
+DMS_HD uint32_t follow(const P& p, const Grid& g, uint32_t* path, Cell c, uint32_t j) {
+  for (int it = 0; it < kFewSteps && !(c.w & kEnd); ++it) {
+    const int64_t v = c.x + g.nx * c.y + g.sxy * c.z;
+    if (is_landmark(v)) {
+      const uint32_t w = claim(path + v * P::K + c.k, kLink | j);
+      if (!(w & kEnd)) return w;
+    }
+    p.step(g, path, v, c);
+  }
+  return c.w;
+}
+// walk j's end, or 0.  Its result becomes what it leads to at every link, for
+// those that link here: chains shorten while they are followed.
+DMS_HD uint32_t end_of(volatile uint32_t* results, int64_t j) {
+  uint32_t w = results[j];
+  for (int it = 0; it < kFewLinks && w & kLink && !(w & kEnd); ++it) results[j] = w = results[w & ~kLink];
+  return w & kEnd ? w : 0;
 }
 
 }  // namespace dms

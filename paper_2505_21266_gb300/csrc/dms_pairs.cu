@@ -324,9 +324,10 @@ __global__ void __launch_bounds__(kBrickThreads) resolve_paths(const P p, uint32
   }
 }
 
-__device__ __forceinline__ uint32_t walk_end(const Walk& a, int32_t* dstatus) {
-  if (a.w < kLoop) return a.w & ~kEnd;
-  set_status(dstatus, a.w == kLoop ? DMS_ERR_TIMEOUT : DMS_ERR_ARG);  // bad data
+// the node at a path's end, from its word
+__device__ __forceinline__ uint32_t walk_end(uint32_t w, int32_t* dstatus) {
+  if (w < kLoop) return w & ~kEnd;
+  set_status(dstatus, w == kLoop ? DMS_ERR_TIMEOUT : DMS_ERR_ARG);  // bad data
   return 0;
 }
 // the saddle's record with its weight and ends, live where they differ.  With
@@ -370,83 +371,153 @@ __device__ __forceinline__ void star_ranks(const Grid& g, const uint32_t* __rest
   }
 }
 
+// Few saddles on a large grid (see few_saddles): the words of the landmarks
+// free, then one walk per thread
+template <class P>
+__global__ void clear_landmarks(int64_t n, uint32_t* path) {
+  constexpr int WORDS = kGroup * P::K;  // of a run, consecutive
+  const int64_t words = (n + kRun - 1) / kRun * WORDS;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < words;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = t / WORDS, c = (r * kRun + landmarks_of(r)) * P::K + (t - r * WORDS);
+    if (c < n * P::K) path[c] = kNoMark;
+  }
+}
+template <class P, class S>
+__global__ void __launch_bounds__(256, 8) follow_cells(const P paths, const S starts, int64_t nwalk,
+                                                       uint32_t* path, uint32_t* results) {
+  const Grid g = paths.fields.g;
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (j < nwalk) results[j] = follow(paths, g, path, starts.at(g, j), (uint32_t)j);
+}
+// walk j's first cell: an end of critical edge j / 2, a cofacet of critical
+// triangle j / 2
+struct EdgeEnds {
+  const int64_t* crit1;
+  __device__ __forceinline__ Cell at(const Grid& g, int64_t j) const {
+    const int64_t id = __ldg(crit1 + (j >> 1)), a = id / 7;
+    const int c = j & 1 ? edge_corner((int)(id - a * 7)) : 0;
+    int x, y, z;
+    coords(g, a, x, y, z);
+    return Cell{0, x + (c & 1), y + ((c >> 1) & 1), z + ((c >> 2) & 1), 0};
+  }
+};
+struct TriCofacets {
+  const int64_t* crit2;
+  __device__ __forceinline__ Cell at(const Grid& g, int64_t j) const {
+    const int64_t id = __ldg(crit2 + (j >> 1)), a = id / 12;
+    int x, y, z;
+    int64_t cof[2];
+    coords(g, a, x, y, z);
+    tri_cofacets(g, a, (int)(id - a * 12), x, y, z, cof);
+    const int64_t t = j & 1 ? cof[1] : cof[0];
+    if (t < 0) return Cell{kEnd, 0, 0, 0, 0};  // OUTSIDE
+    const int64_t v = t / 6;
+    coords(g, v, x, y, z);
+    return Cell{0, x, y, z, (int)(t - v * 6)};
+  }
+};
+
+// Where a saddle's two ends come from:
+//   kBricks  walks over the words of the resolved bricks;
+//   kCells   the results of follow_cells; saddles with a long path go to the
+//            list far[0..*far_n);
+//   kFar     as kBricks, the saddles of that list.
+enum Follow { kBricks, kCells, kFar };
+
 // D0: each critical edge's weight (its lexicographic key), its two descending
 // paths.  (Bound by random reads of orders and path words: 32 registers for 64
 // warps an SM; the D0/D2 stage of 1024^3 takes 80.3 ms with 54, 76.6 with 32.)
-template <class F>
-__global__ void __launch_bounds__(256, 8) link_d0(const F fields, const uint32_t* __restrict__ order,
-                                               const int64_t* __restrict__ crit1,
-                                               const int64_t* n_dev, int64_t n_host,
-                                               const uint32_t* __restrict__ path, Tri T,
-                                               uint32_t* live, unsigned int* live_n,
-                                               int32_t* dstatus, bool tag, Nodes nd) {
+template <Follow HOW, class P>
+__global__ void __launch_bounds__(256, 8) link_d0(
+    const P paths, const uint32_t* __restrict__ order, const int64_t* __restrict__ crit1,
+    const int64_t* n_dev, int64_t n_host, const uint32_t* __restrict__ path, Tri T, uint32_t* live,
+    unsigned int* live_n, uint32_t* results, uint32_t* far, unsigned int* far_n, int32_t* dstatus,
+    bool tag, Nodes nd) {
   __shared__ CtaAppend sh;
   const int64_t ne = n_dev ? *n_dev : n_host;
   // CTA-uniform passes: every thread reaches the appends
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < ne;
        base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    bool keep = false;
+    int64_t i = base + threadIdx.x;
+    bool keep = false, longer = false;
     if (i < ne) {
+      if constexpr (HOW == kFar) i = far[i];
       const int64_t id = crit1[i], a = id / 7;
       const int c = edge_corner((int)(id - a * 7));
       Grid g;
       int64_t off;
-      fields.get(a, g, off);
+      paths.fields.get(a, g, off);
       int x, y, z;
       coords(g, a - off, x, y, z);
       const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
       const int64_t b = a + corner_delta(g, c);
-      Walk wa = walk_from<DescPaths<F>>(path, g, a, x, y, z, 0);
-      Walk wb = walk_from<DescPaths<F>>(path, g, b, x + cx, y + cy, z + cz, 0);
+      Walk wa, wb;
+      if constexpr (HOW == kCells) {
+        wa.w = end_of(results, 2 * i);
+        wb.w = end_of(results, 2 * i + 1);
+        longer = !(wa.w & wb.w & kEnd);
+      } else {
+        wa = walk_from<P>(path, g, a, x, y, z, 0);
+        wb = walk_from<P>(path, g, b, x + cx, y + cy, z + cz, 0);
+      }
       const uint32_t oa = __ldg(order + a), ob = __ldg(order + b);
       const bool up = ob > oa;
       uint32_t r, r2;
       star_ranks(g, order, up ? b : a, up ? x + cx : x, up ? y + cy : y, up ? z + cz : z, min(oa, ob),
                  min(oa, ob), r, r2);
-      walk_both<DescPaths<F>>(path, g, off, wa, wb);
-      keep = store_saddle(T, i, ((uint64_t)(oa > ob ? oa : ob) << 4) | r, walk_end(wa, dstatus),
-                          walk_end(wb, dstatus), tag, nd);
+      if constexpr (HOW != kCells) walk_both<P>(path, g, off, wa, wb);
+      if (!longer)
+        keep = store_saddle(T, i, ((uint64_t)(oa > ob ? oa : ob) << 4) | r, walk_end(wa.w, dstatus),
+                            walk_end(wb.w, dstatus), tag, nd);
     }
-    cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+    if constexpr (HOW == kCells) cta_append2(sh, keep, live, live_n, longer, far, far_n, (uint32_t)i);
+    else cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
   }
 }
 
 // D2: each critical triangle's weight (decreasing triangle key), the two dual
 // paths from its cofacets
-template <class F>
-__global__ void __launch_bounds__(256, 8) link_d2(const F fields, const uint32_t* __restrict__ order,
-                                               const int64_t* __restrict__ crit2,
-                                               const int64_t* n_dev, int64_t n_host,
-                                               const uint32_t* __restrict__ path, Tri T,
-                                               uint32_t* live, unsigned int* live_n,
-                                               int32_t* dstatus, bool tag, Nodes nd) {
+template <Follow HOW, class P>
+__global__ void __launch_bounds__(256, 8) link_d2(
+    const P paths, const uint32_t* __restrict__ order, const int64_t* __restrict__ crit2,
+    const int64_t* n_dev, int64_t n_host, const uint32_t* __restrict__ path, Tri T, uint32_t* live,
+    unsigned int* live_n, uint32_t* results, uint32_t* far, unsigned int* far_n, int32_t* dstatus,
+    bool tag, Nodes nd) {
   __shared__ CtaAppend sh;
   const int64_t nt = n_dev ? *n_dev : n_host;
   // CTA-uniform passes: every thread reaches the appends
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < nt;
        base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    bool keep = false;
+    int64_t i = base + threadIdx.x;
+    bool keep = false, longer = false;
     if (i < nt) {
+      if constexpr (HOW == kFar) i = far[i];
       const int64_t id = crit2[i], a = id / 12;
       const int k = (int)(id - a * 12);
       Grid g;
-      int64_t off, cof[2];
-      fields.get(a, g, off);
+      int64_t off;
+      paths.fields.get(a, g, off);
       int x, y, z;
       coords(g, a - off, x, y, z);
-      tri_cofacets(g, a, k, x, y, z, cof);
       Walk wk[2];
+      if constexpr (HOW == kCells) {
+        wk[0].w = end_of(results, 2 * i);
+        wk[1].w = end_of(results, 2 * i + 1);
+        longer = !(wk[0].w & wk[1].w & kEnd);
+      } else {
+        int64_t cof[2];
+        tri_cofacets(g, a, k, x, y, z, cof);
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (cof[j] < 0) {
-          wk[j] = Walk{kEnd, 0, 0, 0};  // no cofacet on that side: OUTSIDE
-        } else {
-          const int64_t v = cof[j] / 6;
-          int vx, vy, vz;
-          coords(g, v - off, vx, vy, vz);
-          wk[j] = walk_from<DualPaths<F>>(path, g, v, vx, vy, vz, (int)(cof[j] - v * 6));
+        for (int j = 0; j < 2; ++j) {
+          if (cof[j] < 0) {
+            wk[j] = Walk{kEnd, 0, 0, 0};  // no cofacet on that side: OUTSIDE
+          } else {
+            const int64_t v = cof[j] / 6;
+            int vx, vy, vz;
+            coords(g, v - off, vx, vy, vz);
+            wk[j] = walk_from<P>(path, g, v, vx, vy, vz, (int)(cof[j] - v * 6));
+          }
         }
       }
       // the key: the order of the highest vertex, the ranks of the others
@@ -470,10 +541,13 @@ __global__ void __launch_bounds__(256, 8) link_d2(const F fields, const uint32_t
       star_ranks(g, order, a + corner_delta(g, ct), x + (ct & 1), y + ((ct >> 1) & 1),
                  z + ((ct >> 2) & 1), om, ol, rm, rl);
       const uint64_t key = ((uint64_t)max(o[0], max(o[1], o[2])) << 8) | (rm << 4) | rl;
-      walk_both<DualPaths<F>>(path, g, off, wk[0], wk[1]);
-      keep = store_saddle(T, i, kMask44 - key, walk_end(wk[0], dstatus), walk_end(wk[1], dstatus), tag, nd);
+      if constexpr (HOW != kCells) walk_both<P>(path, g, off, wk[0], wk[1]);
+      if (!longer)
+        keep = store_saddle(T, i, kMask44 - key, walk_end(wk[0].w, dstatus), walk_end(wk[1].w, dstatus),
+                            tag, nd);
     }
-    cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
+    if constexpr (HOW == kCells) cta_append2(sh, keep, live, live_n, longer, far, far_n, (uint32_t)i);
+    else cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
   }
 }
 
@@ -1145,6 +1219,47 @@ DiagWs carve_diag(void* base, const int64_t* nc, int64_t npath) {
   return w;
 }
 
+// Whether the paths of nsad saddles are followed cell by cell.  The bricks cost
+// the same however few the saddles are, 21 ns per 1000 vertices; the walks
+// break even at 0.03 saddles per vertex on every grid that is large enough for
+// the depth of their chains to be hidden.  D0/D2 stage by bricks and by cells:
+// 1024^3 mixtures of 2e-7, 2.3e-3, 9e-3, 3.0e-2 and 5.6e-2 saddles per vertex
+// 23.2 / 3.7, 25.4 / 7.4, 30.5 / 17.8, 41.4 / 41.9 and 50.9 / 63.3 ms; 512^3,
+// 1.3e-6, 4e-3, 1.6e-2, 3.2e-2 and 5.9e-2: 3.28 / 1.64, 3.82 / 2.06, 4.64 / 3.61,
+// 5.86 / 5.87 and 8.18 / 9.65; 384^3, 8e-6 and 2.8e-2: 1.60 / 1.42 and 2.86 /
+// 2.84; 256^3, 1e-5 and 2.3e-2: 0.72 / 0.99 and 1.25 / 1.31.
+constexpr int64_t kFewGrid = 1 << 25, kFewPer = 32;
+bool few_saddles(int64_t nsad, int64_t n) { return n >= kFewGrid && nsad <= n / kFewPer; }
+
+// the saddles' weights and ends: link(kernel, n) launches one of the three
+template <class P, class S, class L, class K>
+int link_saddles(DiagWs& w, const P& paths, const S& starts, uint32_t node0, int64_t nsad, const L& link,
+                 K* bricks, K* cells, K* far, cudaStream_t s) {
+  const Grid& g = paths.fields.g;
+  const bool few = few_saddles(nsad, g.n);
+  if (few) {
+    const int64_t nb = (g.n / kRun + 1) * kGroup * P::K / 256 + 1;
+    clear_landmarks<P><<<(unsigned)std::min<int64_t>(nb, 1 << 16), 256, 0, s>>>(g.n, w.path); count_launch();
+  }
+  if (paths.n > 0) {
+    mark_ends<<<(unsigned)((paths.n + 255) / 256), 256, 0, s>>>(paths.ends, nullptr, paths.n, node0, w.path); count_launch();
+  }
+  if (few) {
+    follow_cells<<<(unsigned)((2 * nsad + 255) / 256), 256, 0, s>>>(
+        paths, starts, 2 * nsad, w.path, reinterpret_cast<uint32_t*>(w.rb.ka)); count_launch();
+    link(cells, nsad);
+    unsigned int h = 0;
+    DMS_CUDA_OK(cudaMemcpyAsync(&h, w.ctr + kCtrFar, sizeof(h), cudaMemcpyDeviceToHost, s));
+    DMS_CUDA_OK(cudaStreamSynchronize(s));
+    if (h == 0) return launch_status();
+    bricks = far;
+    nsad = h;
+  }
+  resolve_paths<<<(unsigned)brick_count<P>(g.nx, g.ny, g.nz), kBrickThreads, 0, s>>>(paths, w.path); count_launch();
+  link(bricks, nsad);
+  return launch_status();
+}
+
 // the saddles that the rounds left live, if any, in sorted order
 int finish_sorted(DiagWs& w, Tri T, cudaStream_t s) {
   unsigned int h = 0;
@@ -1406,6 +1521,7 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
   }
   const int TB = 256;
   auto nb = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, (n + TB - 1) / TB); };
+  uint32_t* const results = reinterpret_cast<uint32_t*>(w.rb.ka);  // (two words per saddle)
 
   // ---- D0
   DMS_CUDA_OK(cudaMemsetAsync(w.ctr, 0, kCtrWords * sizeof(unsigned int), s));
@@ -1415,12 +1531,14 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
   }
   w.nd.immortal = kNone;  // every minimum but the global one can die
   if (nc[1] > 0) {
-    const DescPaths<OneField> paths{OneField{g}, desc, crit0, nullptr, nc[0]};
-    mark_ends<<<nb(nc[0]), TB, 0, s>>>(crit0, nullptr, nc[0], 0, w.path); count_launch();
-    resolve_paths<<<(unsigned)brick_count<DescPaths<OneField>>(g.nx, g.ny, g.nz), kBrickThreads, 0, s>>>(
-        paths, w.path); count_launch();
-    link_d0<<<nb(nc[1]), TB, 0, s>>>(OneField{g}, order, crit1, nullptr, nc[1], w.path, w.T0, w.live0,
-                                     w.ctr + kCtrLive, dstatus, pairing == 0, w.nd); count_launch();
+    using Paths = DescPaths<OneField>;
+    const Paths paths{OneField{g}, desc, crit0, nullptr, nc[0]};
+    auto link = [&](auto kernel, int64_t n) {
+      kernel<<<nb(n), TB, 0, s>>>(paths, order, crit1, nullptr, n, w.path, w.T0, w.live0, w.ctr + kCtrLive,
+                                  results, w.live1, w.ctr + kCtrFar, dstatus, pairing == 0, w.nd); count_launch();
+    };
+    DMS_TRY(link_saddles(w, paths, EdgeEnds{crit1}, 0u, nc[1], link, link_d0<kBricks, Paths>, link_d0<kCells, Paths>,
+                         link_d0<kFar, Paths>, s));
   }
   int st = pairing == 1 ? run_selfcorrecting(w, w.T0, std::max<int64_t>(nc[0], 1), s, dstatus)
                         : run_pairing(w, w.T0, nc[1], std::max<int64_t>(nc[0], 1), s, dstatus, true);
@@ -1433,14 +1551,14 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
   init_nodes_d2<<<nb(nc[3] + 1), TB, 0, s>>>(D, order, crit3, nc[3], w.nd); count_launch();
   w.nd.immortal = 0;  // OUTSIDE
   if (nc[2] > 0) {
-    const DualPaths<OneField> paths{OneField{g}, rec, crit3, nullptr, nc[3]};
-    if (nc[3] > 0) {
-      mark_ends<<<nb(nc[3]), TB, 0, s>>>(crit3, nullptr, nc[3], 1, w.path); count_launch();
-    }
-    resolve_paths<<<(unsigned)brick_count<DualPaths<OneField>>(g.nx, g.ny, g.nz), kBrickThreads, 0, s>>>(
-        paths, w.path); count_launch();
-    link_d2<<<nb(nc[2]), TB, 0, s>>>(OneField{g}, order, crit2, nullptr, nc[2], w.path, w.T2, w.live0,
-                                     w.ctr + kCtrLive, dstatus, pairing == 0, w.nd); count_launch();
+    using Paths = DualPaths<OneField>;
+    const Paths paths{OneField{g}, rec, crit3, nullptr, nc[3]};
+    auto link = [&](auto kernel, int64_t n) {
+      kernel<<<nb(n), TB, 0, s>>>(paths, order, crit2, nullptr, n, w.path, w.T2, w.live0, w.ctr + kCtrLive,
+                                  results, w.live1, w.ctr + kCtrFar, dstatus, pairing == 0, w.nd); count_launch();
+    };
+    DMS_TRY(link_saddles(w, paths, TriCofacets{crit2}, 1u, nc[2], link, link_d2<kBricks, Paths>, link_d2<kCells, Paths>,
+                         link_d2<kFar, Paths>, s));
   }
   st = pairing == 1 ? run_selfcorrecting(w, w.T2, nc[3] + 1, s, dstatus)
                     : run_pairing(w, w.T2, nc[2], nc[3] + 1, s, dstatus, true);
@@ -1882,8 +2000,9 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   mark_ends<<<G, TB, 0, s>>>(crit[0], cnt_dev + 0, 0, 0, w.path); count_launch();
   resolve_paths<<<(unsigned)bricks0, kBrickThreads, 0, s>>>(Desc{mf, desc, crit[0], cnt_dev + 0, 0}, w.path); count_launch();
   w.nd.immortal = kNone;
-  link_d0<<<G, TB, 0, s>>>(mf, order, crit[1], cnt_dev + 1, 0, w.path, w.T0, w.live0, w.ctr + kCtrLive,
-                           dstatus, true, w.nd); count_launch();
+  link_d0<kBricks, Desc><<<G, TB, 0, s>>>(Desc{mf, desc, crit[0], cnt_dev + 0, 0}, order, crit[1], cnt_dev + 1,
+                                          0, w.path, w.T0, w.live0, w.ctr + kCtrLive, nullptr, nullptr, nullptr,
+                                          dstatus, true, w.nd); count_launch();
   DMS_TRY(rounds(w.T0, cnt_dev + 0, 0));
   DMS_TRY(write(0, w.T0, crit[0], crit[1], cnt_dev + 1, d0, pair_offsets, pair_totals + 0, fcount));
 
@@ -1894,8 +2013,9 @@ int launch_diagram_batch(const float* f, const uint32_t* order, const uint8_t* d
   brick_table<<<1, 32, 0, s>>>(ft, Dual::LX, Dual::LY, Dual::LZ, brick0); count_launch();
   resolve_paths<<<(unsigned)bricks2, kBrickThreads, 0, s>>>(Dual{mf, rec, crit[3], cnt_dev + 3, 0}, w.path); count_launch();
   w.nd.immortal = 0;  // OUTSIDE, shared by all fields
-  link_d2<<<G, TB, 0, s>>>(mf, order, crit[2], cnt_dev + 2, 0, w.path, w.T2, w.live0, w.ctr + kCtrLive,
-                           dstatus, true, w.nd); count_launch();
+  link_d2<kBricks, Dual><<<G, TB, 0, s>>>(Dual{mf, rec, crit[3], cnt_dev + 3, 0}, order, crit[2], cnt_dev + 2,
+                                          0, w.path, w.T2, w.live0, w.ctr + kCtrLive, nullptr, nullptr, nullptr,
+                                          dstatus, true, w.nd); count_launch();
   DMS_TRY(rounds(w.T2, cnt_dev + 3, 1));
   DMS_TRY(write(2, w.T2, crit[2], crit[3], cnt_dev + 2, d2, pair_offsets + (nfields + 1), pair_totals + 1,
                 fcount + (nfields + 1)));
@@ -2014,7 +2134,7 @@ __global__ void __launch_bounds__(256) link2d_d0(Grid2d g, const uint32_t* __res
     const uint64_t w = ((uint64_t)(oa > ob ? oa : ob) << 4) |
                        local_rank2d(g, order, oa > ob ? a : b, oa > ob ? ob : oa);
     walk_both<DescPaths2d>(path, g3, 0, wa, wb);
-    keep = store_saddle(T, i, w, walk_end(wa, dstatus), walk_end(wb, dstatus), false, nd);
+    keep = store_saddle(T, i, w, walk_end(wa.w, dstatus), walk_end(wb.w, dstatus), false, nd);
   }
   cta_append2(sh, keep, live, live_n, false, live, live_n, (uint32_t)i);
 }
@@ -2051,7 +2171,7 @@ __global__ void __launch_bounds__(256) link2d_d1(Grid2d g, const int64_t* __rest
                                    : Walk{kEnd, 0, 0, 0};
       }
       walk_both<DualPaths2d>(path, g3, 0, wk[0], wk[1]);
-      keep = store_saddle(T, i, kMask44 - T.s[i].w, walk_end(wk[0], dstatus), walk_end(wk[1], dstatus),
+      keep = store_saddle(T, i, kMask44 - T.s[i].w, walk_end(wk[0].w, dstatus), walk_end(wk[1].w, dstatus),
                           false, nd);
     }
   }

@@ -22,6 +22,7 @@ enum : int {
   kCtrForest = 2,    // saddles of the spanning forest
   kCtrChanged = 3,   // (self-correcting pairing)
   kCtrBig = 4,       // saddles left to the device-wide sorted finish (batch)
+  kCtrFar = 5,       // saddles whose paths are long (see kCells)
   kCtrRound = 8,     // three live counts in turn, of the grid's rounds
   kCtrLeft = 11,     // saddles left live by the exact rounds
   kCtrBarrier = 12,

@@ -73,6 +73,30 @@ void ends_of(const Grid& g, const uint32_t* path, const int64_t* cells, int64_t 
   }
 }
 
+// the same cell by cell, no brick resolved, the walks in the order given: as
+// one after the other, then their links
+template <class P>
+void cell_ends_of(const P& p, const Grid& g, uint32_t* path, const int64_t* cells, int64_t n,
+                  const int64_t* order, uint32_t* out) {
+  for (int64_t i = 0; i < 2 * n; ++i) {
+    const int64_t j = order[i], at = cells[j], v = at / P::K;
+    const Cell c = at < 0 ? Cell{kEnd, 0, 0, 0, 0}
+                          : Cell{0, (int)(v % g.nx), (int)(v / g.nx % g.ny), (int)(v / g.sxy), (int)(at % P::K)};
+    out[j] = follow(p, g, path, c, (uint32_t)j);
+  }
+  for (int64_t j = 0; j < 2 * n; ++j) out[j] = end_of(out, j);
+}
+template <class P>
+std::vector<uint32_t> marked(const Grid& g, const int64_t* ends, int64_t n, uint32_t node0) {
+  // (what no one wrote: anything)
+  std::vector<uint32_t> path(g.n * P::K);
+  for (size_t c = 0; c < path.size(); ++c) path[c] = (uint32_t)(c * 2654435761u);
+  for (int64_t v = 0; v < g.n; ++v)
+    for (int k = 0; k < P::K && is_landmark(v); ++k) path[v * P::K + k] = kNoMark;
+  for (int64_t i = 0; i < n; ++i) path[ends[i]] = kEnd | (uint32_t)(i + node0);
+  return path;
+}
+
 Grid grid(int64_t nx, int64_t ny, int64_t nz) { return Grid{nx, ny, nz, nx * ny * nz, nx * ny}; }
 
 }  // namespace
@@ -80,23 +104,24 @@ Grid grid(int64_t nx, int64_t ny, int64_t nz) { return Grid{nx, ny, nz, nx * ny 
 extern "C" {
 
 // ends: the cells of the nodes.  starts: two cells per saddle (-1: outside).
-// out: the words of their ends.
+// order: cell by cell, the walks in this order (null: over the bricks).  out:
+// the words of their ends.
 int host_desc_ends(const uint8_t* desc, int64_t nx, int64_t ny, int64_t nz, const int64_t* ends,
-                   int64_t nends, const int64_t* starts, int64_t n, uint32_t* out) {
+                   int64_t nends, const int64_t* starts, int64_t n, const int64_t* order, uint32_t* out) {
   const Grid g = grid(nx, ny, nz);
-  std::vector<uint32_t> path(g.n, 0u);
-  for (int64_t i = 0; i < nends; ++i) path[ends[i]] = kEnd | (uint32_t)i;
+  std::vector<uint32_t> path = marked<DescPaths<OneField>>(g, ends, nends, 0);
   const DescPaths<OneField> p{OneField{g}, desc, ends, nullptr, nends};
+  if (order) return cell_ends_of(p, g, path.data(), starts, n, order, out), 0;
   resolve(p, g, path.data());
   ends_of<std::decay_t<decltype(p)>>(g, path.data(), starts, n, out);
   return 0;
 }
 int host_dual_ends(const uint64_t* rec, int64_t nx, int64_t ny, int64_t nz, const int64_t* ends,
-                   int64_t nends, const int64_t* starts, int64_t n, uint32_t* out) {
+                   int64_t nends, const int64_t* starts, int64_t n, const int64_t* order, uint32_t* out) {
   const Grid g = grid(nx, ny, nz);
-  std::vector<uint32_t> path(g.n * 6, 0u);
-  for (int64_t i = 0; i < nends; ++i) path[ends[i]] = kEnd | (uint32_t)(i + 1);
+  std::vector<uint32_t> path = marked<DualPaths<OneField>>(g, ends, nends, 1);
   const DualPaths<OneField> p{OneField{g}, rec, ends, nullptr, nends};
+  if (order) return cell_ends_of(p, g, path.data(), starts, n, order, out), 0;
   resolve(p, g, path.data());
   ends_of<std::decay_t<decltype(p)>>(g, path.data(), starts, n, out);
   return 0;

@@ -1,6 +1,7 @@
 """The v-path words and walks of the kernels (csrc/dms_bricks.cuh, built for
 the host) on the CPU: on the oracle's gradients of grids that span several
-bricks, every saddle's two walks end where the oracle's triplets say; and a walk
+bricks, every saddle's two walks end where the oracle's triplets say, over the
+bricks' words and cell by cell; and a walk
 over words that loop from brick to brick (no gradient gives them, inconsistent
 arrays of a caller may) ends as a loop after about the hops that the loop has,
 not after as many as the grid has cells, while a valid walk of any length
@@ -20,6 +21,19 @@ from test_walk_schedule import OUTSIDE, _check, _d0_instance, _d2_instance
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_2505_21266_gb300", "csrc")
 END, LOOP = 0x80000000, 0xFFFFFFFE
+
+
+def _ends(fn, src, shape, nodes, cells, turns):
+    """The end words of the walks from cells; turns: cell by cell, in that
+    order (None: over the bricks)."""
+    nz, ny, nx = shape
+    out = np.zeros(len(cells), np.uint32)
+    assert fn(ctypes.c_void_p(src.ctypes.data), *(ctypes.c_int64(v) for v in (nx, ny, nz)),
+              ctypes.c_void_p(nodes.ctypes.data), ctypes.c_int64(len(nodes)),
+              ctypes.c_void_p(cells.ctypes.data), ctypes.c_int64(len(cells) // 2),
+              ctypes.c_void_p(None if turns is None else turns.ctypes.data),
+              ctypes.c_void_p(out.ctypes.data)) == 0
+    return out
 
 
 def _build(d, name):
@@ -64,21 +78,21 @@ def _fields():
 
 @pytest.mark.parametrize("k", range(5))
 @pytest.mark.parametrize("kind", ["d0", "d2"])
-def test_walks_reach_the_oracle_ends(lib, gradient, kind, k):
+@pytest.mark.parametrize("how", ["bricks", "cells", "cells reversed", "cells shuffled"])
+def test_walks_reach_the_oracle_ends(lib, gradient, how, kind, k):
     f = list(_fields())[k]
-    nz, ny, nx = f.shape
     desc, rec = gradient(f)
     saddles, starts, _, nodes, trip = (_d0_instance if kind == "d0" else _d2_instance)(f)
     assert saddles
     nodes = np.array(sorted(nodes), np.int64)
     cells = np.array([-1 if isinstance(s, tuple) else s for s in starts], np.int64)
-    out = np.zeros(len(cells), np.uint32)
+    turns = np.arange(len(cells), dtype=np.int64)
+    if how == "cells reversed":
+        turns = turns[::-1].copy()
+    if how == "cells shuffled":
+        np.random.default_rng(k).shuffle(turns)
     fn, src = (lib.host_desc_ends, desc) if kind == "d0" else (lib.host_dual_ends, rec)
-    args = [ctypes.c_void_p(src.ctypes.data), *(ctypes.c_int64(v) for v in (nx, ny, nz)),
-            ctypes.c_void_p(nodes.ctypes.data), ctypes.c_int64(len(nodes)),
-            ctypes.c_void_p(cells.ctypes.data), ctypes.c_int64(len(saddles)),
-            ctypes.c_void_p(out.ctypes.data)]
-    assert fn(*args) == 0
+    out = _ends(fn, src, f.shape, nodes, cells, None if how == "bricks" else turns)
     node = out.astype(np.int64) - END
     assert (node >= 0).all()
     if kind == "d0":
@@ -103,3 +117,27 @@ def test_a_long_walk_reaches_its_end(lib, rows):
     end = np.zeros(1, np.uint32)
     assert lib.host_long_walk(rows, 0, end.ctypes.data) == 32 * rows + 1
     assert int(end[0]) == END + 7
+
+
+@pytest.mark.parametrize("turns,done", [([0, 1, 2, 3], [3]), ([3, 2, 1, 0], [0, 1, 2, 3]),
+                                        ([1, 3, 0, 2], [3])])
+def test_long_paths_wait_for_the_bricks(lib, turns, done):
+    """A slope of 6000 vertices: cell by cell a walk from its top is too long,
+    and so is any that joins it (from 4000, behind one that got down to 1900,
+    too); from the top behind a walk that reached the end it is not.  Over the
+    bricks all reach it.  Round a ring (no gradient) a walk ends as too long."""
+    shape, n = (2, 2, 6000), 24000
+    desc = np.full(n, 7, np.uint8)  # to x - 1
+    desc[0] = 15
+    for row in (6000, 12000, 18000):
+        desc[row] = 11 if row == 18000 else (8 if row == 6000 else 9)  # -y-z, -y, -z
+    nodes = np.zeros(1, np.int64)
+    cells = np.array([5990, 5999, 4000, 70], np.int64)
+    turns = np.array(turns, np.int64)
+    assert (_ends(lib.host_desc_ends, desc, shape, nodes, cells, None) == END).all()
+    out = _ends(lib.host_desc_ends, desc, shape, nodes, cells, turns)
+    assert [j for j in range(4) if out[j] == END] == done and all(out[j] in (0, END) for j in range(4))
+    desc[3000:3002] = 0, 7  # 3000 -> 3001 -> 3000
+    out = _ends(lib.host_desc_ends, desc, shape, nodes, np.array([3000, 3500], np.int64), np.arange(2))
+    assert (out == 0).all()
+    assert (_ends(lib.host_desc_ends, desc, shape, nodes, np.array([3000, 3500], np.int64), None) == LOOP).all()
