@@ -11,7 +11,9 @@
 //
 // Work layout: a CTA owns a TX x TY x ZC block of ANCHORS and streams it along
 // z.  Per slab z, in two phases of tasks of 32 that the warps draw from a
-// counter (corrections differ in length):
+// counter (corrections differ in length), over what of the tile lies in the
+// grid (over whole tiles, grids thin in x or y paid for the rest: 4096 x 2 x
+// 4096 smooth 9.7 ms, now 3.1; 4096 x 4096 x 2 13.6, now 6.7):
 //   1. every vertex of the slab reads the kinds of the 14 edges whose higher
 //      end it may be: desc, or an entry in one of four lists by how long its
 //      correction takes; the records two slabs down, final by now, are written
@@ -34,9 +36,12 @@
 // the correction inlined four times and its loops unrolled by the compiler a
 // 512^3 noise field took 37 ms instead of 17.  The correction's lanes advance
 // in step (any_lane); left to diverge in nested loops it took 75 ms.
-// Measured (GB300): 1024^3 mixture with noise 123.5 -> 88 ms, 512^3 quantised
-// noise 17.7 -> 16.9 ms, 64^3 and 24^3 mixtures 0.28 -> 0.11 and 0.19 -> 0.05
+// Measured (GB300): 1024^3 mixture with noise 124 -> 90 ms, 512^3 quantised
+// noise 17.8 -> 16.9 ms, 64^3 and 24^3 mixtures 0.28 -> 0.11 and 0.19 -> 0.06
 // ms, against ProcessLowerStars run queue by queue with one thread per vertex.
+// It is slower than that on noise in grids of fewer than 24 vertices in x, or
+// 9 to 16 in y, whose slabs have too few vertices for a CTA's warps: 2048 x
+// 2048 x 8 11.2 against 9.1 ms, 1024 x 1024 x 16 3.8 against 3.1.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -71,7 +76,10 @@ constexpr int ctas_of(int ty) { return ty == 24 ? 3 : (ty == 32 ? 2 : 4); }
 // us each where corrections are many), are the time.  24^3 and 64^3 mixtures:
 // 51 and 107 us against 392 and 832 us in tiles of 24 rows and chunks of 32
 // slabs; above the line the taller tile's smaller halo wins (203 x 131 x 77
-// noise, 2.0 M vertices: 434 us against 551 us).
+// noise, 2.0 M vertices: 434 us against 551 us).  Grids of up to kSmallTY rows
+// take these tiles at any size, which they fill (2048 x 8 x 2048 noise 6.4 ms,
+// in tiles of 24 rows 8.5; from 9 rows on the tall tile is faster: 300 x 10 x
+// 1500 noise 1.19 against 1.56 ms).
 constexpr int kSmallTY = 8;
 constexpr int64_t kSmallGrid = (int64_t)1 << 20;
 
@@ -81,6 +89,15 @@ template <int PARTS>
 constexpr int part_of_type(int t) {
   return PARTS == 1 ? 0 : (t < 3 ? 0 : 1);
 }
+
+// rows of equal length, numbered through: row of number i < 1156 of at most 34
+// columns ((i * inv) >> 16 is exact for i * cols < 2^16)
+struct Rows {
+  int cols, rows, n, inv;
+  Rows() = default;
+  __device__ __forceinline__ Rows(int c, int r) : cols(c), rows(r), n(c * r), inv(65536 / c + 1) {}
+  __device__ __forceinline__ int row(int i) const { return (i * inv) >> 16; }
+};
 
 // shared memory of a CTA working on tiles of TX x TY anchors.  The order
 // field is staged slab by slab in windows of WY rows x WX columns: with TMA
@@ -121,6 +138,7 @@ struct Smem {
   unsigned int task[2];      // the next task of the two phases
   unsigned int counts[4];
   uint32_t one;    // the number 1 (see add_if_less)
+  Rows verts, anchors;  // what of the tile lies in the grid
   long long tile;  // batched kernel: the tile this CTA works on
 };
 
@@ -475,16 +493,24 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
     return (int)__shfl_sync(0xFFFFFFFFu, t, 0);
   };
 
+  // tasks are drawn over what of the tile lies in the grid: its vertices, and
+  // its anchors from -1 on
+  if (tid == 0) {
+    const int vx = (int)min(g.nx - x0, (int64_t)TX + 1), vy = (int)min(g.ny - y0, (int64_t)TY + 1);
+    sm.verts = Rows(vx, vy);
+    sm.anchors = Rows(vx + 1, vy + 1);
+  }
+
   // the rule for 64 anchors (their edges of one part) of the slab with window
   // b0 (its neighbours' bm, bp) and record slab rz (the one below: rzm)
-  constexpr int kRuleTasks = (S::FN + 63) / 64 * PARTS;
   auto rule_task = [&](int task, int bm, int b0, int bp, int rz, int rzm, uint32_t one) {
     const uint32_t *wm = sm.win[bm], *w0 = sm.win[b0], *wp = sm.win[bp];
+    const Rows anchors = sm.anchors;
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
       const int a = (PARTS == 2 ? task >> 1 : task) * 64 + k * 32 + lane;
-      if (a >= S::FN) return;
-      const int lx = a % S::FX - 1, ly = a / S::FX - 1;
+      if (a >= anchors.n) return;
+      const int row = anchors.row(a), lx = a - row * anchors.cols - 1, ly = row - 1;
       if (PARTS == 2 && (task & 1))
         apply_rule<PARTS - 1, S, PARTS>(sm, wm, w0, wp, lx, ly, rz, rzm, one);
       else
@@ -493,12 +519,12 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
   };
 
   // desc of 32 vertices of slab z, or their entries in the lists of `fz`
-  constexpr int kVertTasks = (S::VN + 31) / 32;
   auto vert_task = [&](int task, int64_t z, int rz, int rzm, int fz) {
     const int i = task * 32 + lane;
-    const int lx = i % (TX + 1), ly = i / (TX + 1);
+    const Rows verts = sm.verts;
+    const int ly = verts.row(i), lx = i - ly * verts.cols;
     int cls = -1;
-    if (i < S::VN && x0 + lx < g.nx && y0 + ly < g.ny) {
+    if (i < verts.n) {
       const uint32_t w = vertex_kinds(sm, lx, ly, rz, rzm);
       const uint32_t b0 = w & 0x5555555u, b1 = (w >> 1) & 0x5555555u, empty = b0 & ~b1;
       if (empty != 0 && (b1 != 0 || (empty & (empty - 1)) != 0)) {
@@ -528,7 +554,8 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
     const int e = first + lane;
     const bool on = e < count;
     const int i = on ? sm.list[cls >> 1][(cls & 1) ? S::VN - 1 - e : e] : 0;
-    const int lx = i % (TX + 1), ly = i / (TX + 1);
+    const Rows verts = sm.verts;
+    const int ly = verts.row(i), lx = i - ly * verts.cols;
     const int at = (ly + 2) * S::WX + lx + S::XOFF;
     TileStar<S> star{sm, at, (ly + 2) * S::RX + lx + 2, b0, rz, rzm};
     uint32_t lm = 0;
@@ -547,13 +574,13 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
 
   // writes out a row of anchors of slab zw in record slab r (all of whose
   // vertices' slabs are done) and clears the row's words for the slab that
-  // takes them over; the rows past TY are the halo's, only cleared
-  constexpr int kFlushTasks = TY + 3;
+  // takes them over; the last three are the halo's, only cleared
   auto flush_task = [&](int row, int64_t zw, int r) {
-    const int ry = row < TY ? row + 2 : (row == TY + 2 ? TY + 2 : row - TY);
+    const int frows = min(sm.verts.rows, TY);
+    const int ry = row < frows ? row + 2 : (row == frows + 2 ? TY + 2 : row - frows);
     uint32_t* hi = &sm.hi[r][ry * S::RX];
     const int64_t gx = x0 + lane, gy = y0 + row;
-    if (row < TY && zw >= z0 && zw < zend && gy < g.ny && gx < g.nx) {
+    if (row < frows && zw >= z0 && zw < zend && gx < g.nx) {
       uint32_t l = sm.lo[0][r][ry * S::RX + 2 + lane], h = hi[2 + lane];
       if constexpr (PARTS == 2) l |= sm.lo[PARTS - 1][r][ry * S::RX + 2 + lane];
       // simplices that leave the grid are absent
@@ -600,10 +627,11 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
 #pragma unroll 1
     for (int k = j < 0 ? 0 : (j + 2 <= J ? 1 : 2); k < 2; ++k) ok = land() && ok;
     if (j >= 1) {
-      const int first = in ? 0 : kVertTasks;
-      for (int t = next_task(1) + first; t < kVertTasks + kFlushTasks; t = next_task(1) + first) {
-        if (t < kVertTasks) vert_task(t, z, rz, rzm, fz);
-        else flush_task(t - kVertTasks, z - 2, rzp);
+      const int vertTasks = (sm.verts.n + 31) / 32, first = in ? 0 : vertTasks;
+      const int all = vertTasks + min(sm.verts.rows, TY) + 3;
+      for (int t = next_task(1) + first; t < all; t = next_task(1) + first) {
+        if (t < vertTasks) vert_task(t, z, rz, rzm, fz);
+        else flush_task(t - vertTasks, z - 2, rzp);
       }
     }
     if (tid < 4) sm.nlist[fz ^ 1][tid] = 0;  // the next slab's; the last slab's are done
@@ -623,7 +651,7 @@ __device__ bool gradient_tile(Smem<TY, TMA, PARTS>& sm, const uint32_t* __restri
     const int per = listed >= NT ? 32 : max(4, (listed + NT / 32 - 1) / (NT / 32));
     const int t3 = ((int)nl.w + per - 1) / per, t2 = t3 + ((int)nl.z + per - 1) / per;
     const int t1 = t2 + ((int)nl.y + per - 1) / per, tasks = t1 + ((int)nl.x + per - 1) / per;
-    const int all = tasks + (j < jlast ? kRuleTasks : 0);
+    const int all = tasks + (j < jlast ? (sm.anchors.n + 63) / 64 * PARTS : 0);
     const uint32_t one = *(volatile uint32_t*)&sm.one;
     for (int t = next_task(0); t < all; t = next_task(0)) {
       if (t >= tasks) {
@@ -811,7 +839,7 @@ int launch_single(const uint32_t* order, const Grid& g, uint8_t* desc, uint64_t*
   const int64_t tx = (g.nx + TX - 1) / TX, ty = (g.ny + TY - 1) / TY;
   const int64_t cap = (int64_t)sms * per_sm, tiles = tx * ty;
   int64_t nzc;
-  if (TY == kSmallTY) {
+  if (g.n <= kSmallGrid) {
     // a small grid: the CTAs' slabs one after the other are the time, so as
     // few slabs each as fill the GPU once
     nzc = std::max<int64_t>(1, std::min<int64_t>(cap / tiles, g.nz));
@@ -819,10 +847,13 @@ int launch_single(const uint32_t* order, const Grid& g, uint8_t* desc, uint64_t*
     // about 16 waves of resident CTAs, so that the last, partly filled wave
     // costs little, in chunks of at least 32 slabs (each chunk also applies
     // the rule to the slabs below and above it); a grid that such chunks leave under two
-    // waves takes chunks down to 8 slabs
+    // waves takes chunks down to 8 slabs, and one wave where the second would
+    // be nearly empty (300 x 300 x 16 noise, 494 CTAs for 456 places: 0.56 ms
+    // against 0.40 in one wave)
     nzc = std::max<int64_t>(1, std::min<int64_t>((16 * cap + tiles - 1) / tiles, g.nz / 32));
     if (tiles * nzc < 2 * cap)
       nzc = std::max<int64_t>(1, std::min<int64_t>((2 * cap + tiles - 1) / tiles, (g.nz + 7) / 8));
+    if (tiles <= cap && tiles * nzc > cap && tiles * nzc * 4 < cap * 5) nzc = cap / tiles;
   }
   const int zc = (int)((g.nz + nzc - 1) / nzc);
   nzc = (g.nz + zc - 1) / zc;
@@ -885,7 +916,8 @@ int launch_gradient_tiles(const uint32_t* order, const Grid& g, uint8_t* desc, u
 
 int launch_gradient(const uint32_t* order, const Grid& g, uint8_t* desc, uint64_t* rec,
                     int64_t* crit_counts, cudaStream_t s) {
-  return g.n <= kSmallGrid ? launch_gradient_tiles<kSmallTY>(order, g, desc, rec, crit_counts, s)
+  return g.n <= kSmallGrid || g.ny <= kSmallTY
+             ? launch_gradient_tiles<kSmallTY>(order, g, desc, rec, crit_counts, s)
                            : launch_gradient_tiles<24>(order, g, desc, rec, crit_counts, s);
 }
 
