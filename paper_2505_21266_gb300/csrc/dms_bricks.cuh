@@ -365,7 +365,8 @@ DMS_HD void walk_both(Path path, const Grid& g, int64_t off, Walk& a, Walk& b) {
 }
 
 // ---------------------------------------------------------------------------
-// Few saddles on a large grid: paths cell by cell, no brick resolved.
+// Few saddles on a large grid, or a thin one: paths cell by cell, no brick
+// resolved.
 //
 // Walks that meet go on as one.  One vertex in eight is a landmark: the first
 // walk at a cell of it claims the cell's word, a later one stops there with a

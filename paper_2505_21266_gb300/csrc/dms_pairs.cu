@@ -371,7 +371,7 @@ __device__ __forceinline__ void star_ranks(const Grid& g, const uint32_t* __rest
   }
 }
 
-// Few saddles on a large grid (see few_saddles): the words of the landmarks
+// Paths cell by cell (see follow_by_cells): the words of the landmarks
 // free, then one walk per thread
 template <class P>
 __global__ void clear_landmarks(int64_t n, uint32_t* path) {
@@ -1228,23 +1228,37 @@ DiagWs carve_diag(void* base, const int64_t* nc, int64_t npath) {
 // 1.3e-6, 4e-3, 1.6e-2, 3.2e-2 and 5.9e-2: 3.28 / 1.64, 3.82 / 2.06, 4.64 / 3.61,
 // 5.86 / 5.87 and 8.18 / 9.65; 384^3, 8e-6 and 2.8e-2: 1.60 / 1.42 and 2.86 /
 // 2.84; 256^3, 1e-5 and 2.3e-2: 0.72 / 0.99 and 1.25 / 1.31.
-constexpr int64_t kFewGrid = 1 << 25, kFewPer = 32;
-bool few_saddles(int64_t nsad, int64_t n) { return n >= kFewGrid && nsad <= n / kFewPer; }
+//
+// Bricks that reach far outside a thin grid cost nearly what full ones do, so
+// there the walks win at any density that keeps them short.  By bricks and by
+// cells, (z, y, x): 4096 x 4096 x 2 noise 8.7 / 3.4 ms, 4096 x 2 x 4096 6.1 /
+// 3.5, 4096 x 2048 x 4 (bricks four times the grid) 7.0 / 4.8, 2048 x 1024 x 2
+// 1.6 / 0.95; 1024 x 1024 x 2 1.1 / 0.8, 512 x 512 x 2 0.60 / 0.55; 2048 x 2048
+// x 6 (not four times) 5.0 / 4.2; smooth fields, whose walks are long: 2 x 2048
+// x 2048 0.71 / 1.24, 20,000 x 9 x 9 1.2 / 5.6.
+constexpr int64_t kFewGrid = 1 << 25, kFewPer = 32, kThinGrid = 1 << 21, kThinBricks = 4, kThinPer = 64;
+template <class P>
+bool follow_by_cells(int64_t nsad, const Grid& g) {
+  if (2 * nsad >= (int64_t)kLink) return false;
+  const int64_t bricks = brick_count<P>(g.nx, g.ny, g.nz) << (P::LX + P::LY + P::LZ);
+  return (g.n >= kFewGrid && nsad <= g.n / kFewPer) ||
+         (g.n >= kThinGrid && bricks >= kThinBricks * g.n && nsad >= g.n / kThinPer);
+}
 
 // the saddles' weights and ends: link(kernel, n) launches one of the three
 template <class P, class S, class L, class K>
 int link_saddles(DiagWs& w, const P& paths, const S& starts, uint32_t node0, int64_t nsad, const L& link,
                  K* bricks, K* cells, K* far, cudaStream_t s) {
   const Grid& g = paths.fields.g;
-  const bool few = few_saddles(nsad, g.n);
-  if (few) {
+  const bool cells_first = follow_by_cells<P>(nsad, g);
+  if (cells_first) {
     const int64_t nb = (g.n / kRun + 1) * kGroup * P::K / 256 + 1;
     clear_landmarks<P><<<(unsigned)std::min<int64_t>(nb, 1 << 16), 256, 0, s>>>(g.n, w.path); count_launch();
   }
   if (paths.n > 0) {
     mark_ends<<<(unsigned)((paths.n + 255) / 256), 256, 0, s>>>(paths.ends, nullptr, paths.n, node0, w.path); count_launch();
   }
-  if (few) {
+  if (cells_first) {
     follow_cells<<<(unsigned)((2 * nsad + 255) / 256), 256, 0, s>>>(
         paths, starts, 2 * nsad, w.path, reinterpret_cast<uint32_t*>(w.rb.ka)); count_launch();
     link(cells, nsad);
