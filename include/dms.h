@@ -221,8 +221,10 @@ int dms_critical_noalloc(const uint8_t* desc, const uint64_t* rec, dms_dims d, i
  *        dms_critical).
  *   ws   at least dms_diagram_workspace_size(d, n_crit) bytes (it includes
  *        one 32-bit word per tetrahedron id, 24 bytes per vertex).
- * This call synchronises `stream` between pairing rounds (it reads the
- * number of live saddles on the host).
+ * This call synchronises `stream`: it reads on the host how many saddles the
+ * pairing's rounds leave, how many are live between them while those are very
+ * many, and, where paths are followed cell by cell (few saddles on a large
+ * grid, or a thin grid), how many were too long for that.
  */
 size_t dms_diagram_workspace_size(dms_dims d, const int64_t* n_crit);
 int dms_diagram_d0d2(const float* f, const uint32_t* order, const uint8_t* desc,

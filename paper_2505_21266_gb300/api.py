@@ -44,8 +44,9 @@ def _raise_status(v: int, where: str):
 class _Counts:
     """A stage's counts (int64) and, behind them, its device status, so that one
     copy to the host brings both: each read waits for the device and costs about
-    20 us.  On 24^3 three reads in place of six took the path from 784 to 651 us,
-    on 64^3 from 944 to 829."""
+    20 us.  On 24^3 three reads in place of six, beside the two that the pairing
+    makes itself (the saddles its rounds leave, for D0 and for D2), took the path
+    from 784 to 651 us, on 64^3 from 944 to 829."""
 
     def __init__(self, n: int, device):
         self.n = n

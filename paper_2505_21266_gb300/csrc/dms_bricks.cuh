@@ -61,8 +61,9 @@ constexpr uint64_t entry(int e) {
 // 100 instructions per tet and a word per cell written, which noise, whose
 // paths are short, pays back in fewer random reads: D0/D2 stage 64^3 mixture
 // 705 -> 356 us, 128^3 smooth 953 -> 368 us, 16384^2 37.8 -> 30.8 ms, 512^3
-// ties 28.9 -> 25.1 ms, 1024^3 87.7 -> 75.8 ms (of it a dual step as a sum on
-// the cell's word, in place of packed coordinates: 1.5).  Following every cell to its
+// ties 28.9 -> 25.3 ms, 1024^3 87.7 -> 73.5 ms (of it a dual step as a sum on
+// the cell's word, in place of packed coordinates: 1.5, and the walks' loop
+// without a count of the grid's cells: 2).  Following every cell to its
 // end in turn instead of doubling took 147 ms there.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kEnd = 0x80000000u;

@@ -7,7 +7,9 @@
 //    to the virtual OUTSIDE node when the path leaves the grid.  The paths are
 //    first resolved by bricks of the grid in shared memory (every cell learns
 //    where its path leaves the brick, or its extremum), then each saddle hops
-//    from brick to brick.  Triplets whose two ends coincide are dropped.
+//    from brick to brick; few saddles on a large grid, and many on a thin one,
+//    are followed cell by cell (follow_by_cells).  Triplets whose two ends
+//    coincide are dropped.
 // 2. Pairing rounds.  Alg. 1 visits the saddles in increasing order and, with
 //    a union-find whose roots are the oldest extremum of each component,
 //    pairs the saddle with the younger root when it joins two components.
@@ -1587,9 +1589,9 @@ int launch_diagram(const float* f, const uint32_t* order, const uint8_t* desc, c
 // ===========================================================================
 // Batched form: many fields in one pass, nothing synchronising the host.
 // The critical lists hold GLOBAL ids (anchors in the concatenated arrays);
-// every field is traced with its own dims; the pairing runs a fixed number
-// of rounds on the device (sizes read from device memory) and finishes the
-// last few saddles in sorted order in one CTA.  D0 graphs of different
+// every field is traced with its own dims; the pairing's rounds run on the
+// device, which reads the counts, until they end (pair_rounds), and what they
+// leave is finished in sorted order.  D0 graphs of different
 // fields are disjoint; the D2 graphs share the OUTSIDE node, which is older
 // than every maximum, so each field's pairs are those it has alone.
 // ===========================================================================
@@ -1881,7 +1883,10 @@ __global__ void __launch_bounds__(PNT) b_write_pairs(int dim, const FieldTab ft,
 
 }  // namespace
 
-constexpr unsigned int kBatchLarge = 6;  // (live saddles fall to a third per round or faster)
+// rounds of one launch per phase ahead of pair_rounds, which takes whatever is
+// live then: on noise and on mixtures the live saddles fell to a third or less
+// per round, so that six leave a thousandth
+constexpr unsigned int kBatchLarge = 6;
 int diagram_batch_rounds() { return (int)kMaxExactRounds; }
 
 // Workspace of the batched pairing: the DiagWs of the capacities plus the
